@@ -20,10 +20,10 @@
  *             stage (no registers touched)
  *   hist_u8   per-CTA counts -> cluster accumulator (global atomics) -> copied
  *             out by rank 0.  Small shares count into per-warp bins with
- *             shared atomics; large shares count into lane-private 32-bit
- *             counters, which no two lanes of a warp ever share, so random
- *             bytes cause no shared-memory bank conflicts; with one CTA per
- *             SM every warp streams its part through a ring of its own.
+ *             shared atomics; shares from 16 KB count into lane-private
+ *             32-bit counters, which no two lanes of a warp ever share, so
+ *             random bytes cause no shared-memory bank conflicts; with one
+ *             CTA per SM every warp streams its part through a ring of its own.
  *   sum_f32   per-thread float accumulators, warp shuffles, per-CTA partial;
  *             rank 0 adds the partials in rank order in binary64
  *   gemm64    64x64x64 float32 tiles staged into shared memory by TMA bulk
@@ -61,9 +61,10 @@ __device__ __forceinline__ int4 add4(int4 x, int4 y) {
 #define LK_SMEM_WORK (64u * 1024u)     /* histogram counters or GEMM stages   */
 #define LK_SMEM_STREAM (128u * 1024u)  /* streaming stages                    */
 #define LK_SMEM_DYN (LK_SMEM_WORK + LK_SMEM_STREAM)
+#define LK_TC_SMEM (224u * 1024u)      /* P = 1: the tensor-core GEMM and the histogram's table and rings */
 #define LK_STAGES 4u
 #define LK_GEMM_STAGE_FLOATS 8192u     /* one GEMM stage: A rows 16 KB + B tile 16 KB */
-#define LK_HIST_COPIES 2u              /* lane-private counter copies (32 KB each), P = 1 */
+#define LK_HIST_COPIES 1u              /* lane-private counter copies (32 KB each) */
 #define LK_NUM_BARS 8u                 /* mbarriers: one per stage; the tensor-core GEMM's MMA completion in 4-7 */
 #define LK_WARP_BARS (32u * LK_STAGES)  /* then one per stage of each warp's own ring (histogram) */
 #define LK_ALL_BARS (LK_NUM_BARS + LK_WARP_BARS)
@@ -75,7 +76,7 @@ struct SmemCfg {
   static constexpr uint32_t stream_bytes = LK_SMEM_STREAM / P;
   static constexpr uint32_t dyn_bytes = work_bytes + stream_bytes;
   static constexpr uint32_t gemm_stages = dyn_bytes / (LK_GEMM_STAGE_FLOATS * 4u);   /* 6 or 3 */
-  static constexpr uint32_t hist_copies = LK_HIST_COPIES / P;
+  static constexpr uint32_t hist_copies = LK_HIST_COPIES;
   static_assert(gemm_stages <= LK_NUM_BARS, "one mbarrier per stage");
 };
 
@@ -225,6 +226,7 @@ __device__ __forceinline__ void direct(const uint4* in, uint64_t beg, uint64_t t
 #pragma unroll
   for (int i = 0; i < K; ++i) {
     const uint64_t v = threadIdx.x + (uint64_t)i * T;
+    q[i] = make_uint4(0, 0, 0, 0);
     if (v < total) q[i] = ld_stream(in + beg + v);
   }
 #pragma unroll
@@ -254,6 +256,7 @@ __device__ __forceinline__ bool body_add(const lk_slot& d, int r, int S, unsigne
 #pragma unroll
     for (uint32_t i = 0; i < LK_DIRECT_ADD; ++i) {
       const uint64_t v = beg + threadIdx.x + (uint64_t)i * T;
+      x[i] = y[i] = make_int4(0, 0, 0, 0);
       if (v < end) {
         x[i] = ld_stream(a + v);
         y[i] = ld_stream(b + v);
@@ -371,14 +374,9 @@ __device__ __forceinline__ void combine_sum(const lk_slot& d, const float* parti
 /* ---- uint8 histogram ---------------------------------------------------- */
 /* Shares below this many bytes per CTA use per-warp bins, whose set-up and
  * read-out are cheap; larger shares use the conflict-free lane-private path
- * (measured crossover on GB300: a 28 KB share counts in 2.5 us lane-private
+ * (measured crossover on GB300: a 28 KB share counts in 2.2 us lane-private
  * against 2.9 us in per-warp bins; a 7 KB share in 1.9 against 1.7 us). */
 #define LK_HIST_SMALL_BYTES (16u * 1024u)
-/* With one CTA per SM, shares from this many bytes per CTA stream through
- * one ring per warp (measured on GB300 over 152 CTAs: from 0.4 MB per CTA
- * 3-4 % faster at 256 threads and 14 % at 512; below 0.2 MB 1-4 % slower,
- * where the CTA's single ring needs fewer copies and waits). */
-#define LK_HIST_WARP_BYTES (256u * 1024u)
 
 __device__ __forceinline__ void count4_warp(uint32_t* bins, uint32_t w) {
   atomicAdd(&bins[w & 0xffu], 1u);
@@ -421,54 +419,92 @@ __device__ __forceinline__ void hist_zero(uint32_t* sh, uint32_t words) {
   for (uint32_t i = threadIdx.x; i < words / 4; i += blockDim.x) z[i] = make_uint4(0, 0, 0, 0);
 }
 
-/* ---- histogram of a large share, one CTA per SM ------------------------- */
-/* Counters: word 64 v + 32 c + lane counts bin v for one lane of copy c
- * (two copies, 64 KB).  A bin's row is 256 bytes, so the byte offset of
- * bin v is v << 8: one byte permute moves byte b of a loaded word into
- * bits 8..15, and an add of the lane's base makes the address.  Lane l
- * still touches only bank l.  The 16 bytes of one vector: every address is
- * formed before the first reduction, so the reductions issue back to back. */
+/* ---- histogram of a share with one CTA per SM --------------------------- */
+/* Counters: word 64 v + 32 c + lane counts bin v for one lane of copy c, in a
+ * 64 KB table that starts on a 64 KB boundary of the shared window.  A bin's
+ * row is 256 bytes, so byte 1 of a counter's address is the bin itself and
+ * the other three bytes belong to the lane: one byte permute of the loaded
+ * word and the lane's base makes each address (no add).  Lane l only touches
+ * bank l.  The 16 bytes of one vector: every address is formed before the
+ * first reduction, so the reductions issue back to back.
+ * What bounds it is the shared-memory pipe: 512 bytes of input cost 16 warp
+ * reductions, a 128-bit read per lane (4 wavefronts) and the TMA write of the
+ * same bytes (4), 24 clocks or 21.3 bytes a clock.  Measured per SM: 20.4 with
+ * HBM idle (38 CTAs), 19 on 152 CTAs (3 x 1 GiB: 5.80 TB/s; with a permute
+ * and an add per address, and two copies to clear and read, 16.6 and 5.23).
+ * Loads straight into registers instead of through the ring: 21.1 on 38 CTAs,
+ * but 5.24 TB/s on 152, too few bytes in flight.  A second copy of the
+ * counters only adds clearing and read-out. */
 __device__ __forceinline__ void count16_row(uint32_t lane_addr, uint4 q) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
   uint32_t a[16];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) a[4 * i + b] = lane_addr + __byte_perm(w[i], 0u, 0x4404u | ((uint32_t)b << 4));
+    for (int b = 0; b < 4; ++b) a[4 * i + b] = __byte_perm(w[i], lane_addr, 0x7604u | ((uint32_t)b << 4));
 #pragma unroll
   for (int j = 0; j < 16; ++j) asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(a[j]) : "memory");
 }
 
-/* Thread v (< 256) adds row v (both copies, 32 lanes each); each 8-thread
- * phase of the 128-bit loads starts at thread-dependent columns and so
- * touches all 32 banks once. */
-__device__ __forceinline__ uint32_t hist_row_readout(const uint32_t* sh, uint32_t v) {
-  const uint4* rw = reinterpret_cast<const uint4*>(sh + v * 64u);
+/* Shared-memory offset (from dsm) of the counter table, and of warp w's ring:
+ * three quarters of the rings follow the table (96 KB), the others end where
+ * it starts (32 KB). */
+__device__ __forceinline__ uint32_t hist_table_off(const unsigned char* dsm) {
+  return ((smem_addr(dsm) + 0xffffu) & ~0xffffu) - smem_addr(dsm);
+}
+#define LK_HIST_TABLE 65536u
+
+/* Clear the counters of the copies in use (the first 128 * copies bytes of
+ * each 256-byte row). */
+template <uint32_t COPIES>
+__device__ __forceinline__ void hist_row_zero(unsigned char* tbl) {
+  constexpr uint32_t per_row = COPIES * 8u;   /* 16-byte words */
+  for (uint32_t i = threadIdx.x; i < 256u * per_row; i += blockDim.x)
+    *reinterpret_cast<uint4*>(tbl + (i / per_row) * 256u + (i % per_row) * 16u) = make_uint4(0, 0, 0, 0);
+}
+
+/* Thread v (< 256) adds row v (32 lanes of each copy); each 8-thread phase
+ * of the 128-bit loads starts at thread-dependent columns and so touches all
+ * 32 banks once. */
+template <uint32_t COPIES>
+__device__ __forceinline__ uint32_t hist_row_readout(const unsigned char* tbl, uint32_t v) {
+  constexpr uint32_t per_row = COPIES * 8u;
+  const uint4* rw = reinterpret_cast<const uint4*>(tbl + v * 256u);
   uint32_t tot = 0;
 #pragma unroll
-  for (uint32_t j = 0; j < 16; ++j) {
-    const uint4 q = rw[(j + v) & 15u];
+  for (uint32_t j = 0; j < per_row; ++j) {
+    const uint4 q = rw[(j + v) & (per_row - 1u)];
     tot += (q.x + q.y) + (q.z + q.w);
   }
   return tot;
 }
 
 /* Every warp streams its own contiguous part of the CTA's share [beg, end)
- * (16-byte vectors) through a private ring of LK_STAGES stages -- its slice
- * of the streaming region -- which its lane 0 fills with TMA bulk copies and
- * all its lanes await on the warp's own mbarriers (bars[LK_NUM_BARS + 4 w
- * + s], phase bits LK_NUM_BARS + s of `phase`, which every lane of the warp
- * keeps alike).  A warp never waits for another between chunks (with one
- * ring per CTA, warps stalled about a fifth of their cycles at the per-chunk
- * barrier: random bytes make their counting times uneven).  Returns false,
- * on every thread alike, if a stage did not arrive before the deadline. */
-template <int P, bool YIELD>
+ * (16-byte vectors) through a private ring of LK_STAGES stages (4 KB each at
+ * 256 threads; six or eight smaller stages in the same memory were 10-25 %
+ * slower, stages that are no multiple of 2 KB 11 %), which its
+ * lane 0 fills with TMA bulk copies and all its lanes await on the warp's own
+ * mbarriers (bars[LK_NUM_BARS + 4 w + s], phase bits LK_NUM_BARS + s of
+ * `phase`, which every lane of the warp keeps alike).  A warp never waits for
+ * another between chunks (with one ring per CTA, warps stalled about a fifth
+ * of their cycles at the per-chunk barrier: random bytes make their counting
+ * times uneven).  The first loads are issued before `before_count` runs on
+ * the whole CTA (it clears the counters), so their latency covers it.
+ * Returns false, on every thread alike, if a stage did not arrive before the
+ * deadline. */
+template <int P, bool PAIRS, bool YIELD, class F>
 __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg, uint64_t end, unsigned char* dsm,
-                                                  uint64_t* bars, uint32_t& phase, uint32_t lane_addr, Pace pace) {
-  static_assert(P == 1, "the counter rows take the whole 64 KB work region of one CTA per SM");
+                                                  uint64_t* bars, uint32_t& phase, uint32_t lane_addr, Pace pace,
+                                                  F&& before_count) {
+  static_assert(P == 1, "the counter rows need one CTA per SM's shared memory");
   const uint32_t W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t stage_vec = SmemCfg<P>::stream_bytes / W / LK_STAGES / 16u;
-  uint4* ring = reinterpret_cast<uint4*>(dsm + SmemCfg<P>::work_bytes) + (size_t)warp * LK_STAGES * stage_vec;
+  const uint32_t quarter = (W + 3u) / 4u;                   /* rings before the table */
+  const uint32_t ring_bytes = 32768u / quarter;
+  const uint32_t stage_vec = ring_bytes / LK_STAGES / 16u;
+  const uint32_t tbl = hist_table_off(dsm);
+  const uint32_t ring_off = warp < 3u * quarter ? tbl + LK_HIST_TABLE + warp * ring_bytes
+                                                : tbl - 32768u + (warp - 3u * quarter) * ring_bytes;
+  uint4* ring = reinterpret_cast<uint4*>(dsm + ring_off);
   uint64_t* wb = bars + LK_NUM_BARS + warp * LK_STAGES;
   uint64_t wbeg, wend;
   share(end - beg, (int)warp, (int)W, wbeg, wend);
@@ -477,9 +513,11 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
   /* the warp's part, its ring slice and barriers, and the farthest counter
    * address any byte can form (row 255 of this lane and copy) */
   if (!LK_INB(wbeg <= wend && wend <= end, LK_OOB_SHARE) ||
-      !LK_INB((size_t)(warp + 1) * LK_STAGES * stage_vec * 16u <= SmemCfg<P>::stream_bytes &&
+      !LK_INB(tbl >= 32768u && ring_off + LK_STAGES * stage_vec * 16u <= LK_TC_SMEM &&
+                  (ring_off >= tbl + LK_HIST_TABLE || ring_off + LK_STAGES * stage_vec * 16u <= tbl) &&
                   LK_NUM_BARS + (warp + 1) * LK_STAGES <= LK_ALL_BARS, LK_OOB_STREAM_SMEM) ||
-      !LK_INB(lane_addr - smem_addr(dsm) + 0xff00u + 4u <= SmemCfg<P>::work_bytes, LK_OOB_HIST_COUNTER))
+      !LK_INB(((lane_addr >> 8) & 0xffu) == 0 && lane_addr - smem_addr(dsm) >= tbl &&
+                  lane_addr - smem_addr(dsm) + 0xff00u + 4u <= tbl + LK_HIST_TABLE, LK_OOB_HIST_COUNTER))
     wend = wbeg;
   const uint64_t total = wend - wbeg;
   const uint64_t nch = (total + stage_vec - 1) / stage_vec;
@@ -511,20 +549,73 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
     fence_proxy_async_smem();     /* earlier generic shared accesses before async writes */
     for (uint64_t ch = 0; ch < nch && ch < LK_STAGES; ++ch) issue(ch);
   }
-  bool failed = false;
+  __syncwarp();
+  bool failed = !before_count();
+  auto refill = [&](uint64_t ch) {   /* every lane has read chunk ch: its stage takes chunk ch + LK_STAGES */
+    __syncwarp();
+    if (lane == 0 && ch + LK_STAGES < nch) {
+      /* token bucket as deep as the ring: chunk k >= LK_STAGES no earlier
+       * than t_first + (k - LK_STAGES + 1) chunks' worth of time */
+      if (rate) sleep_until(t_first + (ch + 1) * (uint64_t)stage_vec * 16u * 1000u / rate);
+      if (YIELD) yield.hold();
+      fence_proxy_async_smem();
+      issue(ch + LK_STAGES);
+    }
+  };
+  auto arrived = [&](uint64_t ch) {   /* warp-uniform */
+    return __all_sync(0xffffffffu, mbar_wait(&wb[ch % LK_STAGES], parity(ch), deadline));
+  };
   uint64_t ch = 0;
-  for (; ch < nch; ++ch) {
-    const uint32_t st = (uint32_t)(ch % LK_STAGES);
-    const bool ok = mbar_wait(&wb[st], parity(ch), deadline);
-    if (!__all_sync(0xffffffffu, ok)) {
+  /* At most four warps (stages of 8 KB): whole chunks, in pairs of 2 KB
+   * batches (four vectors a lane), the next batch loaded before the current
+   * one's 64 reductions are issued (they are ordered asm, so loads placed
+   * after them would wait for them), across the stage wait too.  With few
+   * warps nothing else covers those latencies (128 threads: 4.65 -> 5.29
+   * TB/s over 3 x 1 GiB); eight warps cover them for each other and lose to
+   * the longer code (256 threads: 5.88 -> 5.72). */
+  const uint64_t nfull = stage_vec % 512u == 0 ? total / stage_vec : 0;
+  if (PAIRS && nfull && !failed) {   /* PAIRS: kernels of at most 256 threads, which have the registers */
+    uint4 q0[4], q1[4];
+    auto load4 = [&](uint4 (&q)[4], const uint4* s0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) q[i] = s0[lane + 32 * i];
+    };
+    auto count4 = [&](const uint4 (&q)[4]) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) count16_row(lane_addr, q[i]);
+    };
+    failed = !arrived(0);
+    load4(q0, ring);   /* a failed wait's bytes are not counted */
+    for (; ch < nfull && !failed; ++ch) {
+      const uint4* s0 = ring + (size_t)(ch % LK_STAGES) * stage_vec;
+      load4(q1, s0 + 128);
+      count4(q0);
+      for (uint32_t v = 256; v < stage_vec; v += 256) {
+        load4(q0, s0 + v);
+        count4(q1);
+        load4(q1, s0 + v + 128);
+        count4(q0);
+      }
+      if (ch + 1 < nfull) {
+        if (!arrived(ch + 1)) {
+          failed = true;
+          refill(ch++);   /* as after a counted chunk: LK_STAGES chunks from ch on are issued */
+          break;
+        }
+        load4(q0, ring + (size_t)((ch + 1) % LK_STAGES) * stage_vec);
+      }
+      count4(q1);
+      refill(ch);
+    }
+  }
+  for (; ch < nch && !failed; ++ch) {
+    if (!arrived(ch)) {
       failed = true;
       break;
     }
     const uint64_t v0 = wbeg + ch * stage_vec;
     const uint32_t cnt = (uint32_t)((wend - v0) < stage_vec ? (wend - v0) : stage_vec);
-    const uint4* s0 = ring + (size_t)st * stage_vec;
-    /* four vectors loaded before their 64 reductions: the reductions are
-     * ordered asm, so loads placed after them would wait for them */
+    const uint4* s0 = ring + (size_t)(ch % LK_STAGES) * stage_vec;
     uint32_t v = lane;
     for (; v + 96 < cnt; v += 128) {
       uint4 q[4];
@@ -534,15 +625,7 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
       for (int i = 0; i < 4; ++i) count16_row(lane_addr, q[i]);
     }
     for (; v < cnt; v += 32) count16_row(lane_addr, s0[v]);
-    __syncwarp();   /* every lane has read the stage before it is refilled */
-    if (lane == 0 && ch + LK_STAGES < nch) {
-      /* token bucket as deep as the ring: chunk k >= LK_STAGES no earlier
-       * than t_first + (k - LK_STAGES + 1) chunks' worth of time */
-      if (rate) sleep_until(t_first + (ch + 1) * (uint64_t)stage_vec * 16u * 1000u / rate);
-      if (YIELD) yield.hold();
-      fence_proxy_async_smem();
-      issue(ch + LK_STAGES);
-    }
+    refill(ch);
   }
   /* a failed wait leaves the copies issued after it in flight: let them land */
   const uint64_t issued = failed ? (ch + LK_STAGES < nch ? ch + LK_STAGES : nch) : nch;
@@ -594,7 +677,7 @@ __device__ __forceinline__ bool hist_out_ready(const HistSink& sink, uint64_t de
   return s_ready != 0;
 }
 
-template <int P>
+template <int P, bool PAIRS>
 __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsigned char* dsm, uint64_t* bars,
                                           uint32_t& phase, Pace pace, HistSink sink) {
   const uint64_t nv = d.n >> 4;
@@ -605,27 +688,29 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
   const uint32_t T = blockDim.x, W = T / 32, lane = threadIdx.x & 31;
   uint32_t* sh = reinterpret_cast<uint32_t*>(dsm);
   const uint8_t* xb = reinterpret_cast<const uint8_t*>(d.in0);
+  const uint4* in = reinterpret_cast<const uint4*>(d.in0);
   bool ok = true;
   const uint64_t total = end - beg;
-  uint32_t* acc = sink.acc;
-  if (sink.zero) {
-    acc = reinterpret_cast<uint32_t*>(d.out);
-    if (r == 0) {
-      /* the counters' targets start at zero; the others add once they see it */
-      if (sink.prev_done && !hist_out_ready(HistSink{nullptr, const_cast<uint64_t*>(sink.prev_done), sink.seq - 1,
-                                                     nullptr},
-                                            pace.deadline))
-        return false;
-      for (uint32_t v = threadIdx.x; v < 256; v += T) acc[v] = 0;
-      __syncthreads();
-      if (threadIdx.x == 0) st_release_gpu(sink.zero, sink.seq);
-    }
-  }
+  uint32_t* acc = sink.zero ? reinterpret_cast<uint32_t*>(d.out) : sink.acc;
+  /* rank 0 of a sink with a clear word: the counts' targets start at zero;
+   * the others add once they see it */
+  auto clear_out = [&]() -> bool {
+    if (!sink.zero || r != 0) return true;
+    if (sink.prev_done && !hist_out_ready(HistSink{nullptr, const_cast<uint64_t*>(sink.prev_done), sink.seq - 1,
+                                                   nullptr},
+                                          pace.deadline))
+      return false;
+    for (uint32_t v = threadIdx.x; v < 256; v += T) acc[v] = 0;
+    __syncthreads();
+    if (threadIdx.x == 0) st_release_gpu(sink.zero, sink.seq);
+    return true;
+  };
   if (total * 16 < LK_HIST_SMALL_BYTES) {
+    if (!clear_out()) return false;
     hist_zero(sh, W * 256);
     __syncthreads();
     uint32_t* bins = sh + (threadIdx.x >> 5) * 256;
-    ok = stream<1, false, P>(reinterpret_cast<const uint4*>(d.in0), nullptr, beg, end, dsm + SmemCfg<P>::work_bytes, bars, phase,
+    ok = stream<1, false, P>(in, nullptr, beg, end, dsm + SmemCfg<P>::work_bytes, bars, phase,
                           pace, [&](uint64_t, uint32_t cnt, const uint4* s0, const uint4*) {
                             for (uint32_t v = threadIdx.x; v < cnt; v += T) {
                               const uint4 q = s0[v];
@@ -646,71 +731,74 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
     return ok && ready;
   }
   if constexpr (P == 1) {
-    if (total * 16 >= LK_HIST_WARP_BYTES) {
-      /* large share, one CTA per SM: rows of 2 x 32 lane-private counters,
-       * warps w and w + 2 share copy w % 2 (their reductions are atomic) */
-      const uint32_t lane_addr = smem_addr(sh) + ((threadIdx.x >> 5) & 1u) * 128u + lane * 4u;
-      hist_zero(sh, 256u * 64u);
+    /* one CTA per SM: rows of lane-private counters, all warps of a copy
+     * share its words (their reductions are atomic) */
+    constexpr uint32_t copies = LK_HIST_COPIES;
+    unsigned char* tbl = dsm + hist_table_off(dsm);
+    const uint32_t lane_addr = smem_addr(tbl) + ((threadIdx.x >> 5) % copies) * 128u + lane * 4u;
+    auto prepare = [&]() -> bool {
+      hist_row_zero<copies>(tbl);
+      const bool cleared = clear_out();
       __syncthreads();
-      ok = pace.gate ? hist_warp_streams<P, true>(reinterpret_cast<const uint4*>(d.in0), beg, end, dsm, bars, phase,
-                                                  lane_addr, pace)
-                     : hist_warp_streams<P, false>(reinterpret_cast<const uint4*>(d.in0), beg, end, dsm, bars, phase,
-                                                   lane_addr, pace);
-      if (tail)
-        for (uint64_t j = nv * 16 + threadIdx.x; j < d.n; j += T)
-          asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(lane_addr + ((uint32_t)xb[j] << 8))
-                       : "memory");
-      const bool ready = hist_out_ready(sink, pace.deadline);
-      for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
-        const uint32_t tot = hist_row_readout(sh, v);
-        if (tot) atomicAdd(&acc[v], tot);
-      }
-      return ok && ready;
+      return cleared;
+    };
+    ok = pace.gate ? hist_warp_streams<P, PAIRS, true>(in, beg, end, dsm, bars, phase, lane_addr, pace, prepare)
+                   : hist_warp_streams<P, PAIRS, false>(in, beg, end, dsm, bars, phase, lane_addr, pace, prepare);
+    if (tail)
+      for (uint64_t j = nv * 16 + threadIdx.x; j < d.n; j += T)
+        asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(lane_addr + ((uint32_t)xb[j] << 8))
+                     : "memory");
+    const bool ready = hist_out_ready(sink, pace.deadline);
+    for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
+      const uint32_t tot = hist_row_readout<copies>(tbl, v);
+      if (tot) atomicAdd(&acc[v], tot);
     }
-  }
-  /* medium share, or two CTAs per SM: one ring for the CTA; lane-private
-   * 32-bit counters, one set per copy; the W / copies warps of a copy share
-   * its words (their reductions to a word are atomic) */
-  constexpr uint32_t copies = SmemCfg<P>::hist_copies;
-  const uint32_t copy = (threadIdx.x >> 5) % copies;
-  const uint32_t lane_addr = smem_addr(sh + copy * 8192u + lane);
-  hist_zero(sh, copies * 8192u);
-  __syncthreads();
-  ok = stream<1, false, P>(reinterpret_cast<const uint4*>(d.in0), nullptr, beg, end, dsm + SmemCfg<P>::work_bytes, bars, phase,
-                        pace, [&](uint64_t, uint32_t cnt, const uint4* s0, const uint4*) {
-                          /* four vectors loaded before their 64 reductions: the
-                           * reductions are ordered asm, so loads placed after
-                           * them would wait for them */
-                          uint32_t v = threadIdx.x;
-                          for (; v + 3 * T < cnt; v += 4 * T) {
-                            uint4 q[4];
+    return ok && ready;
+  } else {
+    /* two CTAs per SM: one ring for the CTA; lane-private 32-bit counters,
+     * shared by the CTA's warps (their reductions to a word are atomic) */
+    if (!clear_out()) return false;
+    constexpr uint32_t copies = SmemCfg<P>::hist_copies;
+    const uint32_t copy = (threadIdx.x >> 5) % copies;
+    const uint32_t lane_addr = smem_addr(sh + copy * 8192u + lane);
+    hist_zero(sh, copies * 8192u);
+    __syncthreads();
+    ok = stream<1, false, P>(in, nullptr, beg, end, dsm + SmemCfg<P>::work_bytes, bars, phase,
+                          pace, [&](uint64_t, uint32_t cnt, const uint4* s0, const uint4*) {
+                            /* four vectors loaded before their 64 reductions: the
+                             * reductions are ordered asm, so loads placed after
+                             * them would wait for them */
+                            uint32_t v = threadIdx.x;
+                            for (; v + 3 * T < cnt; v += 4 * T) {
+                              uint4 q[4];
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) q[i] = s0[v + i * T];
+                              for (int i = 0; i < 4; ++i) q[i] = s0[v + i * T];
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                              count4_lane(lane_addr, q[i].x);
-                              count4_lane(lane_addr, q[i].y);
-                              count4_lane(lane_addr, q[i].z);
-                              count4_lane(lane_addr, q[i].w);
+                              for (int i = 0; i < 4; ++i) {
+                                count4_lane(lane_addr, q[i].x);
+                                count4_lane(lane_addr, q[i].y);
+                                count4_lane(lane_addr, q[i].z);
+                                count4_lane(lane_addr, q[i].w);
+                              }
                             }
-                          }
-                          for (; v < cnt; v += T) {
-                            const uint4 q = s0[v];
-                            count4_lane(lane_addr, q.x);
-                            count4_lane(lane_addr, q.y);
-                            count4_lane(lane_addr, q.z);
-                            count4_lane(lane_addr, q.w);
-                          }
-                        });
-  if (tail)
-    for (uint64_t j = nv * 16 + threadIdx.x; j < d.n; j += T)
-      asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(lane_addr + ((uint32_t)xb[j] << 7)) : "memory");
-  const bool ready = hist_out_ready(sink, pace.deadline);
-  for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
-    const uint32_t tot = hist_readout<P>(sh, v);
-    if (tot) atomicAdd(&acc[v], tot);
+                            for (; v < cnt; v += T) {
+                              const uint4 q = s0[v];
+                              count4_lane(lane_addr, q.x);
+                              count4_lane(lane_addr, q.y);
+                              count4_lane(lane_addr, q.z);
+                              count4_lane(lane_addr, q.w);
+                            }
+                          });
+    if (tail)
+      for (uint64_t j = nv * 16 + threadIdx.x; j < d.n; j += T)
+        asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(lane_addr + ((uint32_t)xb[j] << 7)) : "memory");
+    const bool ready = hist_out_ready(sink, pace.deadline);
+    for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
+      const uint32_t tot = hist_readout<P>(sh, v);
+      if (tot) atomicAdd(&acc[v], tot);
+    }
+    return ok && ready;
   }
-  return ok && ready;
 }
 
 /* Rank 0: copy the accumulator out and return it to zero for reuse. */
@@ -815,7 +903,6 @@ __device__ __forceinline__ uint32_t gemm_row_split(uint64_t tiles, int S) {
  * the epilogue's row exchange once the MMAs have read them.  TMEM: all 512
  * columns (four blocks of 128), allocated for the body and freed on every
  * path out of it. */
-#define LK_TC_SMEM (224u * 1024u)
 #define LK_TC_STAGES 3u
 #define LK_TC_MMA_BAR 4u             /* bars 4-7: MMA completion of (half, buffer) 2 h + b */
 #define LK_TC_OPS (96u * 1024u)

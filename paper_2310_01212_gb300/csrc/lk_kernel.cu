@@ -372,7 +372,7 @@ __device__ __forceinline__ int run_body(const lk_slot& d, int r, int S, unsigned
     case LK_OP_SUM_F32:
       ok = body_sum<P, (MAXT <= 256 && P == 1)>(d, r, S, dsm, bars, phase, deadline, red, partial_out);
       break;
-    case LK_OP_HIST_U8: ok = body_hist<P>(d, r, S, dsm, bars, phase, deadline, hist); break;
+    case LK_OP_HIST_U8: ok = body_hist<P, (MAXT <= 256)>(d, r, S, dsm, bars, phase, deadline, hist); break;
     case LK_OP_GEMM64_F32:
       ok = body_gemm<(MAXT <= 256 && P == 1), P>(d, r, S, reinterpret_cast<float*>(dsm), bars, phase, deadline, tc);
       break;
@@ -556,7 +556,7 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
       float* pout = parts > 1 ? s_psum + part : &s_part_sum;
       ok = body_sum<P, (MAXT <= 256 && P == 1)>(it, (int)part, (int)parts, dsm, bars, phase, deadline, red, pout);
     } else if (op == LK_OP_HIST_U8) {
-      ok = body_hist<P>(it, (int)part, (int)parts, dsm, bars, phase, deadline,
+      ok = body_hist<P, (MAXT <= 256)>(it, (int)part, (int)parts, dsm, bars, phase, deadline,
                         HistSink{parts > 1 ? s_pbins : my_hist, nullptr, 0, nullptr});
     } else {
       ok = run_body<MAXT, P>(it, (int)part, (int)parts, dsm, bars, phase, red, nullptr, HistSink{}, rate, gate,

@@ -1,0 +1,38 @@
+"""The histogram's counter table and per-warp rings, and the tensor-core GEMM's
+stages and operand buffers, at the sizes where they can go wrong: around the
+small-share cut, one granule more or less than a stage or a ring, every number
+of rings before and after the table (the block size sets it), and tile counts
+around the wrap of the stages and buffers.  The bounds-checking build runs
+them, so every region is checked too.  Histograms are exact; GEMM elements
+stay within 1e-4 sum|a b| of binary64."""
+import numpy as np
+import pytest
+
+from gpu_util import gemm_ok, host, need_gpu, to_dev
+from paper_2310_01212_gb300 import lk, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_ready(native_built):
+    return need_gpu()
+
+
+@pytest.mark.parametrize("threads", [64, 96, 160, 256, 1024])
+def test_hist_share_edges(torch_ready, oracle_lib, threads):
+    torch = torch_ready
+    ring = (32768 // -(-(threads // 32) // 4)) // 64 * 64      # bytes of one warp's ring
+    total = ring * (threads // 32)
+    sizes = [16 * 1024 - 16, 16 * 1024 - 1, 16 * 1024, 16 * 1024 + 1, total // 4 + 16, total - 16, total + 17,
+             3 * total + 16 * 129 + 7]
+    cases = [(x, to_dev(x), torch.full((256,), -1, dtype=torch.int32, device="cuda"))
+             for x in (synth.bytes_uniform(31, i, n) for i, n in enumerate(sizes))]
+    torch.cuda.current_stream().synchronize()
+    with lk.lk_init([1], bounds=True, idle_lease_ns=5_000_000_000, threads_per_cta=threads) as c:
+        hs = [lk.lk_submit(c, 0, lk.LK_OP_HIST_U8, x.size, (dx,), out) for x, dx, out in cases]
+        for h in hs:
+            assert lk.lk_wait(c, h) == lk.LK_OK, lk.lk_device_error(c)
+    for x, _, out in cases:
+        assert np.array_equal(host(out).astype(np.int64), oracle_lib.hist_u8(x)), x.size
+    assert lk.lk_bounds_violations() == (0, 0)
