@@ -65,7 +65,7 @@ __device__ __forceinline__ int4 add4(int4 x, int4 y) {
 #define LK_STAGES 4u
 #define LK_GEMM_STAGE_FLOATS 8192u     /* one GEMM stage: A rows 16 KB + B tile 16 KB */
 #define LK_HIST_COPIES 1u              /* lane-private counter copies (32 KB each) */
-#define LK_NUM_BARS 8u                 /* mbarriers: one per stage; the tensor-core GEMM's MMA completion in 4-7 */
+#define LK_NUM_BARS 8u                 /* mbarriers: one per stage; the tensor-core GEMM's MMA completion in 4, 5 */
 #define LK_WARP_BARS (32u * LK_STAGES)  /* then one per stage of each warp's own ring (histogram) */
 #define LK_ALL_BARS (LK_NUM_BARS + LK_WARP_BARS)
 
@@ -882,33 +882,37 @@ __device__ __forceinline__ uint32_t gemm_row_split(uint64_t tiles, int S) {
  * both rounded to nearest; x - x_hi is exact in float32, and x_hi + x_lo
  * differs from x by at most 2^-16 |x|, so each product a b is formed to
  * within about 2^-15 |a b| (3.1e-5, against the 1e-4 bound; accumulation
- * adds at most 64 float32 roundings).  The A operand stacks A_hi (rows 0-63)
- * on A_lo (rows 64-127) and the B operand B_hi (columns 0-63) on B_lo
- * (64-127), so one chain of four MMAs over K (M = 128, N = 128, K = 16;
- * TMEM rows are lanes 0-127, one to one) yields all four products in a
- * 128 x 128 block D, and
- * C[r][n] = D[r][n] + D[r][n+64] + D[r+64][n] + D[r+64][n+64].
- * Two pipelines, one per half of the CTA (warps 0-3 and 4-7, each with its
- * own named barrier), take alternate tiles.  Each half has two buffers
- * (operands in shared memory, a 128 x 128 block in TMEM, an MMA-completion
- * mbarrier) and alternates between them: it splits tile k into buffer
- * k mod 2, hands it to the tensor core, and finishes tile k-1 (TMEM read-out,
- * row exchange, stores) while those MMAs run, so the tensor core's latency
- * hides behind the epilogue.  The TMA stage ring is shared: tile u sits in
- * stage (u - first) mod 3, and the half that split tile u refills that stage
- * with tile u+3.
- * Shared memory (224 KB): three 32 KB TMA stages of raw tiles (A rows, B) at
- * 0; four 32 KB buffers at 96 KB, two per half: the operands (A' then B',
- * 16 KB each, in the K-major core-matrix layout the descriptors name), then
- * the epilogue's row exchange once the MMAs have read them.  TMEM: all 512
- * columns (four blocks of 128), allocated for the body and freed on every
- * path out of it. */
-#define LK_TC_STAGES 3u
-#define LK_TC_MMA_BAR 4u             /* bars 4-7: MMA completion of (half, buffer) 2 h + b */
-#define LK_TC_OPS (96u * 1024u)
+ * adds at most 129 float32 roundings).  A_lo and A_hi accumulate along K and
+ * B_hi and B_lo lie side by side along N, so eight MMAs (M = 64, N = 128,
+ * K = 16) leave all four products of a tile in a 64 x 128 TMEM block, and
+ * C[r][n] = D[r][n] + D[r][n + 64]: one thread holds both, nothing is
+ * exchanged between threads.  A is K-major and B MN-major (its rows lie along
+ * N in memory), so both operands are split the same way, row by row, with no
+ * transposition: 64 bf16 are the 128 bytes of one swizzled row.
+ *
+ * The CTA's eight warps split tile k into operand buffer k mod 2, one thread
+ * hands it to the tensor core and refills the raw stage, and while those MMAs
+ * run every warp stores its part of tile k-1: one barrier per tile.
+ * What bounds it is HBM: 3 x 2^15 tiles move 6.57 TB/s once booted, as much as
+ * the same loads and stores with neither split nor MMAs (6.63).  One SM alone
+ * (38 CTAs, HBM idle) takes 2,060 clocks a tile, against 2,275 of its share of
+ * HBM: 1,130 for the loads and stores, the rest for the split and the chain
+ * through the MMAs, which take 512 clocks themselves.  Operands stacked along
+ * M and N instead (four MMAs of 128 x 128), B transposed on the way and the
+ * column and row halves added through shared memory moved 5.95 TB/s.  A fifth
+ * stage gains nothing.
+ * Shared memory: four 32 KB TMA stages of raw tiles (A, then B) at 0; two
+ * 32 KB operand buffers (A_hi, A_lo, B_hi, B_lo) from the next 1 KB boundary.
+ * TMEM: 256 columns (two blocks of 128), allocated for the body and freed on
+ * every path out of it. */
+#define LK_TC_STAGES 4u
+#define LK_TC_MMA_BAR 4u            /* bars 4, 5: MMA completion of operand buffer b */
+#define LK_TC_OPS (128u * 1024u)    /* at least: rounded up to 1 KB of the shared window */
+#define LK_TC_COLS 256u
 /* instruction descriptor: D float32 (bits 4-5 = 1), A and B bf16 (bits 7-9,
- * 10-12 = 1), both K-major, N = 128 (bits 17-22 = N/8), M = 128 (bits 24-28 = M/16) */
-#define LK_TC_IDESC ((1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24))
+ * 10-12 = 1), A K-major, B MN-major (bit 16), N = 128 (bits 17-22 = N/8),
+ * M = 64 (bits 24-28 = M/16) */
+#define LK_TC_IDESC ((1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((128u >> 3) << 17) | ((64u >> 4) << 24))
 
 /* (x0, x1) -> bf16 pairs hi = bf16(x), lo = bf16(x - hi), x0 in the low half */
 __device__ __forceinline__ void bf16_split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -917,81 +921,33 @@ __device__ __forceinline__ void bf16_split2(float x0, float x1, uint32_t& hi, ui
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(x1 - h1), "f"(x0 - h0));
 }
 
-/* Eight consecutive k of one operand row (x0: k..k+3, x1: k+4..k+7) -> one
- * 16-byte core-matrix row of hi parts and one of lo parts. */
-__device__ __forceinline__ void bf16_split8(float4 x0, float4 x1, uint4& hi, uint4& lo) {
-  bf16_split2(x0.x, x0.y, hi.x, lo.x);
-  bf16_split2(x0.z, x0.w, hi.y, lo.y);
-  bf16_split2(x1.x, x1.y, hi.z, lo.z);
-  bf16_split2(x1.z, x1.w, hi.w, lo.w);
-}
-
-/* Column e of the 4x4 block q[0..3] (rows k..k+3): the K-chunk of output column n = 4 n4 + e. */
-__device__ __forceinline__ float4 column_of(const float4* q, uint32_t e) {
-  float4 v;
-  v.x = e == 0 ? q[0].x : e == 1 ? q[0].y : e == 2 ? q[0].z : q[0].w;
-  v.y = e == 0 ? q[1].x : e == 1 ? q[1].y : e == 2 ? q[1].z : q[1].w;
-  v.z = e == 0 ? q[2].x : e == 1 ? q[2].y : e == 2 ? q[2].z : q[2].w;
-  v.w = e == 0 ? q[3].x : e == 1 ? q[3].y : e == 2 ? q[3].z : q[3].w;
-  return v;
-}
-
-/* The 128 threads of one half (local index t): split the staged raw tile
- * (A rows at `raw`, B at raw + 16 KB) into an operand buffer.  A core matrix
- * is 8 rows of 8 bf16 (16 bytes); the offset of (row i, K-chunk kc = k/8) is
- * (i/8) 1024 + kc 128 + (i%8) 16 bytes.  The thread-to-chunk maps make each
- * 8-thread phase of a 128-bit access touch eight distinct 16-byte bank
- * groups, on the raw side and on the operand side. */
+/* The 256 threads: split the staged raw tile (A rows at `raw`, B rows at
+ * raw + 16 KB) into an operand buffer (hi rows of A, lo rows of A, hi of B, lo
+ * of B, 8 KB each).  Row i of 64 bf16 takes 128 bytes at i 128, its 16-byte
+ * chunk c at position c ^ (i % 8) (the 128-byte swizzle).  Warp w takes rows
+ * 8 w .. 8 w + 7 of each operand; lane l takes 4-element quarters l % 8 and
+ * l % 8 + 8 of two rows.  An 8-lane phase of the 128-bit reads covers 128
+ * contiguous bytes; the 16 lanes of a 64-bit write cover half a row of two
+ * rows whose numbers differ in bit 2, so in distinct banks. */
 __device__ __forceinline__ void tc_split(const unsigned char* raw, unsigned char* ops, uint32_t t) {
+  const uint32_t w = t >> 5, q = t & 7u, sl = (t >> 3) & 3u;
+  const uint32_t r0 = (sl & 1u) * 4u + (sl >> 1);          /* then r0 + 2 */
+  const unsigned char* src = raw + (8u * w + r0) * 256u + q * 16u;
+  float4 x[8];
 #pragma unroll
-  for (uint32_t q = 0; q < 4; ++q) {                 /* A: 512 chunks of 8 k */
-    const uint32_t c = t + 128u * q;
-    const uint32_t j = c & 7u, s = (c >> 3) & 7u, ig = c >> 6;
-    const uint32_t i = ig * 8u + j, kc = (j + s) & 7u, h = (kc >> 2) & 1u;
-    const unsigned char* src = raw + i * 256u + kc * 32u;
-    /* the half at 16 h first: distinct bank groups across the phase */
-    const float4 xa = *reinterpret_cast<const float4*>(src + h * 16u);
-    const float4 xb = *reinterpret_cast<const float4*>(src + (h ^ 1u) * 16u);
-    uint4 hi, lo;
-    bf16_split8(h ? xb : xa, h ? xa : xb, hi, lo);
-    const uint32_t off = ig * 1024u + kc * 128u + j * 16u;
-    *reinterpret_cast<uint4*>(ops + off) = hi;                         /* A_hi: rows 0-63 */
-    *reinterpret_cast<uint4*>(ops + 8192u + off) = lo;                 /* A_lo: rows 64-127 */
+  for (uint32_t i = 0; i < 8; ++i)                         /* operand i / 4, row r0 + 2 (i / 2 % 2), half i % 2 */
+    x[i] = *reinterpret_cast<const float4*>(src + (i >> 2) * 16384u + ((i >> 1) & 1u) * 512u + (i & 1u) * 128u);
+  const uint32_t dst0 = (8u * w + r0) * 128u + (((q >> 1) ^ r0) << 4) + (q & 1u) * 8u;
+#pragma unroll
+  for (uint32_t i = 0; i < 8; ++i) {
+    /* row + 2: 256 bytes on, chunk position ^ 2; second half: position ^ 4 */
+    unsigned char* dst = ops + (i >> 2) * 16384u + ((dst0 ^ ((((i >> 1) & 1u) << 5) | ((i & 1u) << 6))) + ((i >> 1) & 1u) * 256u);
+    uint2 hi, lo;
+    bf16_split2(x[i].x, x[i].y, hi.x, lo.x);
+    bf16_split2(x[i].z, x[i].w, hi.y, lo.y);
+    *reinterpret_cast<uint2*>(dst) = hi;
+    *reinterpret_cast<uint2*>(dst + 8192u) = lo;
   }
-  {                                                  /* B: 128 blocks of 8 k x 4 n, transposed */
-    const uint32_t n4 = t & 15u, kb = t >> 4;
-    const unsigned char* rb = raw + 16384u;
-    float4 v[8];
-#pragma unroll
-    for (uint32_t m = 0; m < 8; ++m) v[m] = *reinterpret_cast<const float4*>(rb + (8u * kb + m) * 256u + n4 * 16u);
-#pragma unroll
-    for (uint32_t te = 0; te < 4; ++te) {
-      const uint32_t e = (te + (n4 >> 1)) & 3u;      /* rotated: distinct bank groups per phase */
-      const uint32_t n = 4u * n4 + e;
-      uint4 hi, lo;
-      bf16_split8(column_of(v, e), column_of(v + 4, e), hi, lo);
-      const uint32_t off = (n >> 3) * 1024u + kb * 128u + (n & 7u) * 16u;
-      *reinterpret_cast<uint4*>(ops + 16384u + off) = hi;              /* B_hi: rows 0-63 */
-      *reinterpret_cast<uint4*>(ops + 24576u + off) = lo;              /* B_lo: rows 64-127 */
-    }
-  }
-}
-
-/* Barrier of one half (named barrier 1 or 2, 128 threads); the _and form
- * also returns the AND of every participant's `v`, so that all 128 threads
- * take the same branch afterwards. */
-__device__ __forceinline__ void half_sync(uint32_t h) { asm volatile("bar.sync %0, 128;" ::"r"(1u + h) : "memory"); }
-__device__ __forceinline__ bool half_sync_and(uint32_t h, bool v) {
-  uint32_t out;
-  asm volatile(
-      "{\n\t.reg .pred pi, po;\n\t"
-      "setp.ne.u32 pi, %1, 0;\n\t"
-      "bar.red.and.pred po, %2, 128, pi;\n\t"
-      "selp.u32 %0, 1, 0, po;\n\t}"
-      : "=r"(out)
-      : "r"((uint32_t)v), "r"(1u + h)
-      : "memory");
-  return out != 0;
 }
 
 __device__ __forceinline__ bool body_gemm_tc(const lk_slot& d, int r, int S, unsigned char* dsm, uint64_t* bars,
@@ -1000,180 +956,136 @@ __device__ __forceinline__ bool body_gemm_tc(const lk_slot& d, int r, int S, uns
   share(d.n, r, S, beg, end);
   if (!LK_INB(end <= d.n, LK_OOB_SHARE)) end = beg;
   if (beg >= end) return true;
-  const float* A = reinterpret_cast<const float*>(d.in0);
-  const float* B = reinterpret_cast<const float*>(d.in1);
-  float* C = reinterpret_cast<float*>(d.out);
+  const float* A = reinterpret_cast<const float*>(d.in0) + beg * 4096;
+  const float* B = reinterpret_cast<const float*>(d.in1) + beg * 4096;
+  float* C = reinterpret_cast<float*>(d.out) + beg * 4096;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
-  const uint32_t h = warp >> 2, lt = threadIdx.x & 127u;   /* half, index within it */
-  const bool leader = lt == 0;
-  const uint64_t tiles = end - beg;
+  const uint32_t uwarp = __shfl_sync(0xffffffffu, warp, 0);   /* the same, known to be warp-uniform */
+  const uint32_t tiles = (uint32_t)(end - beg);   /* at most 2^28 */
   constexpr uint64_t unit_bytes = 32768u;
   const uint64_t deadline = pace.rate ? pace.deadline + tiles * unit_bytes * 1000u / pace.rate : pace.deadline;
   const uint64_t t_first = pace.rate ? gtime() : 0;
-  auto issue = [&](uint64_t u) {   /* a half's leader, or thread 0 at the start */
-    const uint32_t st = (uint32_t)((u - beg) % LK_TC_STAGES);
+  auto issue = [&](uint32_t u) {   /* one thread: tile u of the share into its stage */
+    const uint32_t st = u % LK_TC_STAGES;
     unsigned char* sa = dsm + st * 32768u;
     fence_proxy_async_smem();
-    if (!LK_INB(u >= beg && u < end, LK_OOB_GEMM_LOAD) || !LK_INB((st + 1) * 32768u <= LK_TC_OPS, LK_OOB_GEMM_SMEM)) {
+    if (!LK_INB(u < tiles, LK_OOB_GEMM_LOAD) || !LK_INB((st + 1) * 32768u <= LK_TC_OPS, LK_OOB_GEMM_SMEM)) {
       mbar_expect_tx(&bars[st], 0u);   /* skipped: the phase completes with no bytes */
       return;
     }
     mbar_expect_tx(&bars[st], 32768u);
-    bulk_g2s(sa, A + u * 4096, 16384u, &bars[st]);
-    bulk_g2s(sa + 16384u, B + u * 4096, 16384u, &bars[st]);
+    bulk_g2s(sa, A + (uint64_t)u * 4096, 16384u, &bars[st]);
+    bulk_g2s(sa + 16384u, B + (uint64_t)u * 4096, 16384u, &bars[st]);
   };
   /* parity of a barrier's k-th completion in this body, from its bit at entry */
-  const uint32_t phase0 = phase;
-  auto parity = [&](uint32_t bar, uint64_t k) { return ((phase0 >> bar) & 1u) ^ (uint32_t)(k & 1u); };
+  auto parity = [&](uint32_t bar, uint32_t k) { return ((phase >> bar) & 1u) ^ (k & 1u); };
   __shared__ uint32_t s_tmem;
-  /* loads issued into each stage so far: a parity wait is only sound one
-   * phase ahead, so a half waits for a stage's next load to be issued (by
-   * the other half, once it consumed the stage's previous tile) before it
-   * waits for that load's phase */
-  __shared__ uint32_t s_issued[LK_TC_STAGES];
   __syncthreads();          /* every stage is free: the previous use ended with a barrier */
-  if (warp == 0) tmem_alloc(&s_tmem, 512);
-  if (threadIdx.x == 0) {
-    for (uint32_t sb = 0; sb < LK_TC_STAGES; ++sb) s_issued[sb] = 0;
-    for (uint64_t u = beg; u < end && u < beg + LK_TC_STAGES; ++u) {
-      issue(u);
-      s_issued[u - beg] = 1;
-    }
+  if (threadIdx.x == 0)
+    for (uint32_t u = 0; u < tiles && u < LK_TC_STAGES; ++u) issue(u);
+  if (warp == 0) {
+    __syncwarp();
+    tmem_alloc(&s_tmem, LK_TC_COLS);
   }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  /* this half's two buffers b: TMEM block dt0 + 128 b, shared memory
-   * ops0 + 32 KB b (operands, then the epilogue's row exchange) */
-  const uint32_t dt0 = s_tmem + 256u * h;
-  unsigned char* ops0 = dsm + LK_TC_OPS + h * 65536u;
-  /* both halves' two buffers inside the shared memory and the 512 TMEM columns */
-  const bool bufs_ok = LK_INB(LK_TC_OPS + (h + 1) * 65536u <= LK_TC_SMEM && 256u * (h + 1) <= 512u, LK_OOB_GEMM_SMEM);
-  /* epilogue: warp quarter q holds D rows 32q..32q+31 (rows 64-127 are the
-   * A_lo products of output rows 0-63) */
-  const uint32_t quarter = warp & 3u;
-  const uint32_t drow = 32u * quarter + lane;
-  /* Tile u, the kk-th of this half, in buffer b = kk & 1: wait for its MMAs,
-   * fold each row's column halves (B_hi and B_lo products) into the buffer,
-   * rows 0-63 at `part`, rows 64-127 at part + 64 x 64 (16-byte chunk c of
-   * row i at position c ^ (i & 7): no bank conflicts on either side), then
-   * add the two parts and store the tile in coalesced 128-bit stores.
-   * Returns false, on all 128 threads alike, if the MMAs did not complete
-   * in time; on return the buffer and its TMEM block are free again. */
-  auto epilogue = [&](uint64_t u, uint64_t kk) -> bool {
-    const uint32_t b = (uint32_t)(kk & 1u), bar = LK_TC_MMA_BAR + 2u * h + b;
-    float* part = reinterpret_cast<float*>(ops0 + 32768u * b);
-    bool done = mbar_wait(&bars[bar], parity(bar, kk >> 1), deadline + 1000000000ull);
-    if (done) {
-      tc_fence_after_sync();
-      float* prow = part + drow * 64u;
-      const uint32_t sw = drow & 7u;
+  const uint32_t tmem = s_tmem;
+  /* both operand buffers inside the shared memory, both blocks in the allocated columns */
+  unsigned char* ops0 = dsm + (((smem_addr(dsm) + LK_TC_OPS + 1023u) & ~1023u) - smem_addr(dsm));
+  const bool bufs_ok =
+      LK_INB((uint32_t)(ops0 - dsm) >= LK_TC_STAGES * 32768u && (uint32_t)(ops0 - dsm) + 2u * 32768u <= LK_TC_SMEM &&
+                 (smem_addr(ops0) & 1023u) == 0 && 2u * 128u <= LK_TC_COLS,
+             LK_OOB_GEMM_SMEM);
+  /* M = 64: row m of the block is TMEM lane 32 (m / 16) + m % 16, so warp w
+   * reads rows 16 (w % 4) .. + 15, columns 32 (w / 4) .. + 31 of both halves
+   * (warps w and w + 4 share a quarter of the lanes).  Of every 8 columns a lane holds
+   * two neighbours in rows lane / 4 and lane / 4 + 8: four lanes write one
+   * 32-byte sector. */
+  const uint32_t crow = 16u * (warp & 3u) + (lane >> 2), ccol = 32u * (warp >> 2) + 2u * (lane & 3u);
+  const uint32_t dt = tmem + ((32u * (warp & 3u)) << 16) + 32u * (warp >> 2);
+  /* Tile u from buffer u & 1: wait for its MMAs, then TMEM -> registers ->
+   * global memory.  False if the MMAs did not complete in time. */
+  auto epilogue = [&](uint32_t u) -> bool {
+    const uint32_t b = u & 1u;
+    if (!mbar_wait(&bars[LK_TC_MMA_BAR + b], parity(LK_TC_MMA_BAR + b, u >> 1), deadline + 1000000000ull)) return false;
+    __syncwarp();
+    tc_fence_after_sync();
+    float v[16], w[16];
+    tmem_ld_16x256b_x4_2(dt + 128u * b, dt + 128u * b + 64u, v, w);
 #pragma unroll
-      for (uint32_t c0 = 0; c0 < 64; c0 += 32) {
-        float v[32], w[32];
-        tmem_ld32(dt0 + 128u * b + ((32u * quarter) << 16) + c0, v);
-        tmem_ld32(dt0 + 128u * b + ((32u * quarter) << 16) + c0 + 64u, w);
+    for (int i = 0; i < 16; ++i) v[i] += w[i];
+    float* c = C + (uint64_t)u * 4096 + crow * 64u + ccol;
+    if (LK_INB(u < tiles && crow + 8u < 64u && ccol + 26u <= 64u, LK_OOB_GEMM_STORE)) {
 #pragma unroll
-        for (uint32_t c = 0; c < 32; c += 4)
-          *reinterpret_cast<float4*>(prow + ((((c0 + c) >> 2) ^ sw) << 2)) =
-              make_float4(v[c] + w[c], v[c + 1] + w[c + 1], v[c + 2] + w[c + 2], v[c + 3] + w[c + 3]);
+      for (uint32_t j = 0; j < 4; ++j) {
+        st_stream(reinterpret_cast<float2*>(c + 8u * j), make_float2(v[4 * j], v[4 * j + 1]));
+        st_stream(reinterpret_cast<float2*>(c + 8u * j + 512u), make_float2(v[4 * j + 2], v[4 * j + 3]));
       }
     }
-    tc_fence_before_sync();         /* these TMEM reads precede this block's next MMAs */
-    if (half_sync_and(h, done)) {
-      float* ct = C + u * 4096;
-#pragma unroll
-      for (uint32_t q = 0; q < 8; ++q) {
-        const uint32_t f = lt + 128u * q, i = f >> 4, c4 = f & 15u, pos = (c4 ^ (i & 7u)) << 2;
-        const float4 x = *reinterpret_cast<const float4*>(part + i * 64u + pos);
-        const float4 y = *reinterpret_cast<const float4*>(part + (i + 64u) * 64u + pos);
-        if (LK_INB(u < end && i * 64u + c4 * 4u + 4u <= 4096u, LK_OOB_GEMM_STORE))
-          st_stream(reinterpret_cast<float4*>(ct + i * 64u + c4 * 4u), make_float4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w));
-      }
-    } else {
-      done = false;
-    }
-    return half_sync_and(h, done);
+    return true;
   };
-  bool ok = true;
-  uint64_t k = 0;                  /* tiles this half has split and handed to the tensor core */
-  for (uint64_t u = beg + h; u < end; u += 2, ++k) {
-    const uint32_t st = (uint32_t)((u - beg) % LK_TC_STAGES);
-    const uint64_t use = (u - beg) / LK_TC_STAGES;   /* completions of stage st before this one */
-    const uint32_t b = (uint32_t)(k & 1u);
-    bool go = true;
-    if (leader) {
-      const volatile uint32_t* iss = s_issued;
-      for (uint32_t it = 0; iss[st] < use + 1; ++it)
-        if ((it & 15) == 15 && gtime() > deadline) {
-          go = false;
-          break;
-        }
-      __threadfence_block();
-      if (go) {
-        go = mbar_wait(&bars[st], parity(st, use), deadline);
-        if (!go) mbar_wait(&bars[st], parity(st, use), deadline + 1000000000ull);   /* let it land */
-      }
-    }
-    if (!half_sync_and(h, go)) {
-      ok = false;
-      break;
-    }
-    mbar_wait(&bars[st], parity(st, use), deadline + 1000000000ull);   /* complete: visibility */
+  bool ok = true;           /* this thread's waits; agreed at each barrier */
+  uint32_t k = 0;           /* tiles handed to the tensor core */
+  for (; k < tiles; ++k) {
+    const uint32_t st = k % LK_TC_STAGES, b = k & 1u;
     unsigned char* ops = ops0 + 32768u * b;
-    tc_split(dsm + st * 32768u, ops, lt);
+    if (ok) ok = mbar_wait(&bars[st], parity(st, k / LK_TC_STAGES), deadline);
+    if (ok) tc_split(dsm + st * 32768u, ops, threadIdx.x);   /* the buffer's last MMAs (tile k-2) have been waited for */
     fence_proxy_async_smem();       /* the operands, written by threads, are read by the tensor core */
-    tc_fence_before_sync();
-    half_sync(h);
-    if (leader) {
-      /* this half has split tile u: its stage takes tile u+3 */
-      if (u + LK_TC_STAGES < end) {
-        if (pace.rate) sleep_until(t_first + (u + 1 - beg) * unit_bytes * 1000u / pace.rate);
-        issue(u + LK_TC_STAGES);
-        __threadfence_block();
-        atomicAdd(&s_issued[st], 1u);
-      }
-      tc_fence_after_sync();
-      const uint32_t ah = smem_addr(ops), bh = ah + 16384u;
-      if (bufs_ok) {
-#pragma unroll
-        for (uint32_t j = 0; j < 4; ++j)
-          umma_f16(dt0 + 128u * b, umma_desc(ah + 256u * j, 128u, 1024u), umma_desc(bh + 256u * j, 128u, 1024u),
-                   LK_TC_IDESC, j > 0);
-      }
-      umma_commit(&bars[LK_TC_MMA_BAR + 2u * h + b]);
-    }
-    /* while the tensor core works on tile u, finish the previous tile */
-    if (k > 0 && !epilogue(u - 2, k - 1)) {
+    tc_fence_before_sync();         /* the TMEM reads of tile k-2 precede this block's next MMAs */
+    if (!__syncthreads_and(ok)) {
       ok = false;
-      ++k;
       break;
     }
+    if (uwarp == 0) {
+      if (elect_one()) {
+        tc_fence_after_sync();
+        if (bufs_ok) {
+          const uint32_t base = smem_addr(ops);
+#pragma unroll
+          for (uint32_t p = 0; p < 2; ++p)                       /* A_lo, then A_hi */
+#pragma unroll
+            for (uint32_t j = 0; j < 4; ++j)                     /* K = 16 each */
+              umma_f16(tmem + 128u * b, umma_desc_sw128(base + (1u - p) * 8192u + 32u * j, 16u, 1024u),
+                       umma_desc_sw128(base + 16384u + 2048u * j, 8192u, 1024u), LK_TC_IDESC, (p | j) != 0);
+        }
+        umma_commit(&bars[LK_TC_MMA_BAR + b]);
+      }
+      __syncwarp();
+    } else if (threadIdx.x == 32 && k + LK_TC_STAGES < tiles) {
+      /* every thread has split tile k: its stage takes tile k + 4 */
+      if (pace.rate) sleep_until(t_first + (k + 1) * unit_bytes * 1000u / pace.rate);
+      issue(k + LK_TC_STAGES);
+    }
+    /* while the tensor core works on tile k, finish the previous tile */
+    if (k > 0) ok = epilogue(k - 1);
   }
-  if (ok && k > 0 && !epilogue(beg + h + 2 * (k - 1), k - 1)) ok = false;
-  /* MMAs of an unfinished tile may still be in flight: the last commit
-   * covers every earlier MMA, so let it complete (bounded) before TMEM is
-   * freed */
-  if (!ok && leader && k > 0) {
-    const uint32_t bar = LK_TC_MMA_BAR + 2u * h + (uint32_t)((k - 1) & 1u);
-    mbar_wait(&bars[bar], parity(bar, (k - 1) >> 1), deadline + 2000000000ull);
+  if (ok) ok = epilogue(tiles - 1);
+  ok = __syncthreads_and(ok);
+  if (!ok && threadIdx.x == 0) {
+    /* copies and MMAs may still be in flight: let them end (bounded) before
+     * the stages and TMEM are given back; the last commit covers every MMA */
+    for (uint32_t u = k; u < tiles && u < k + LK_TC_STAGES; ++u)
+      mbar_wait(&bars[u % LK_TC_STAGES], parity(u % LK_TC_STAGES, u / LK_TC_STAGES), deadline + 1000000000ull);
+    if (k > 0) {
+      const uint32_t bar = LK_TC_MMA_BAR + ((k - 1) & 1u);
+      mbar_wait(&bars[bar], parity(bar, (k - 1) >> 1), deadline + 2000000000ull);
+    }
   }
   tc_fence_before_sync();
-  __syncthreads();          /* both halves done: stages and operand buffers are free */
+  __syncthreads();          /* stages, operand buffers and TMEM are free */
   tc_fence_after_sync();
-  if (warp == 0) tmem_dealloc(s_tmem, 512);
+  if (warp == 0) tmem_dealloc(tmem, LK_TC_COLS);
   /* every thread advances every barrier's phase bit by its completions here */
   if (ok) {
     for (uint32_t sb = 0; sb < LK_TC_STAGES; ++sb) {
-      const uint64_t uses = tiles > sb ? (tiles - sb + LK_TC_STAGES - 1) / LK_TC_STAGES : 0;
-      phase ^= (uint32_t)(uses & 1u) << sb;
+      const uint32_t uses = tiles > sb ? (tiles - sb + LK_TC_STAGES - 1) / LK_TC_STAGES : 0;
+      phase ^= (uses & 1u) << sb;
     }
-    for (uint32_t hh = 0; hh < 2; ++hh) {
-      const uint64_t mine = tiles > hh ? (tiles - hh + 1) / 2 : 0;
-      for (uint32_t bb = 0; bb < 2; ++bb) {
-        const uint64_t commits = mine > bb ? (mine - bb + 1) / 2 : 0;
-        phase ^= (uint32_t)(commits & 1u) << (LK_TC_MMA_BAR + 2u * hh + bb);
-      }
+    for (uint32_t b = 0; b < 2; ++b) {
+      const uint32_t commits = tiles > b ? (tiles - b + 1) / 2 : 0;
+      phase ^= (commits & 1u) << (LK_TC_MMA_BAR + b);
     }
   }
   return ok;

@@ -36,3 +36,21 @@ def test_hist_share_edges(torch_ready, oracle_lib, threads):
     for x, _, out in cases:
         assert np.array_equal(host(out).astype(np.int64), oracle_lib.hist_u8(x)), x.size
     assert lk.lk_bounds_violations() == (0, 0)
+
+
+@pytest.mark.parametrize("S", [1, 2])
+def test_gemm_tile_counts(torch_ready, oracle_lib, S):
+    torch = torch_ready
+    cases = []
+    for i, t in enumerate(list(range(1, 11)) + [17]):
+        A = synth.normal_f32(32, 2 * i, t * 4096).reshape(t, 64, 64)
+        B = synth.normal_f32(32, 2 * i + 1, t * 4096).reshape(t, 64, 64)
+        cases.append((A, B, to_dev(A), to_dev(B), torch.full((t, 64, 64), float("nan"), device="cuda")))
+    torch.cuda.current_stream().synchronize()
+    with lk.lk_init([S], bounds=True, idle_lease_ns=5_000_000_000) as c:
+        hs = [lk.lk_submit(c, 0, lk.LK_OP_GEMM64_F32, A.shape[0], (dA, dB), dC) for A, B, dA, dB, dC in cases]
+        for h in hs:
+            assert lk.lk_wait(c, h) == lk.LK_OK, lk.lk_device_error(c)
+    for A, B, _, _, dC in cases:
+        assert gemm_ok(host(dC), A, B, oracle_lib), A.shape
+    assert lk.lk_bounds_violations() == (0, 0)
