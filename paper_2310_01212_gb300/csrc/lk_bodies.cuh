@@ -360,10 +360,9 @@ __device__ __forceinline__ bool body_sum(const lk_slot& d, int r, int S, unsigne
   return ok;
 }
 
-/* Rank 0: out[0] = partials added in rank order (binary64). */
-__device__ __forceinline__ void combine_sum(const lk_slot& d, const float* partial, int S) {
-  if (threadIdx.x >= 32) return;
-  const uint32_t lane = threadIdx.x;
+/* One warp (lanes `lane` 0-31): out[0] = partials added in rank order (binary64). */
+__device__ __forceinline__ void combine_sum(const lk_slot& d, const float* partial, int S, uint32_t lane) {
+  if (lane >= 32) return;
   double s = 0.0;
   for (int q = (int)lane; q < S; q += 32) s += (double)__ldcg(partial + q);
 #pragma unroll
@@ -640,23 +639,81 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
   return !__syncthreads_or(failed);
 }
 
-/* Where a histogram's counts go.  With `zero` null, every CTA adds its
+/* A persistent CTA's place and its last descriptors, in shared memory (so
+ * that they cost the bodies no registers). */
+struct lk_cta {
+  lk_slot taken[LK_BCAST_DEPTH];   /* descriptor k (0-based) in [k mod D]: the last D taken        */
+  lk_dcluster* dc;                 /* its cluster's device state                                   */
+  uint64_t* done;                  /* its host-visible completion word                             */
+  int32_t cl, rank, size;          /* cluster (-1: none), rank in it, the cluster's CTAs           */
+  uint64_t t_pick[2], t_start[2];  /* stamps of descriptor k in [k mod 2], for the execution log   */
+  uint64_t t_end;                  /* when the last body ended                                     */
+};
+
+/* Where a histogram's counts go.  With `cta` null, every CTA adds its
  * counts into `acc` (zero at rest) and a combine copies it out afterwards
- * (split parts, ordinary launches).  With `zero` set (a descriptor on a
- * cluster), rank 0 clears the output itself and release-stores `seq` into
- * *zero, and every CTA adds its counts straight into the output once it has
- * acquired that word: no combine, and no CTA waits for another at the end.
- * Rank 0 clears only once the cluster's previous descriptor has finished on
- * every CTA (*prev_done >= seq - 1; null when there is none, or the cluster
- * runs one descriptor at a time), so a CTA still writing the same buffer
- * for an earlier descriptor cannot land after the clear: the output ends as
- * the last descriptor's result, as if the descriptors ran one by one. */
+ * (split parts, ordinary launches).  With `cta` set (descriptor `seq` of a
+ * cluster), rank 0 clears the output itself and release-stores seq into the
+ * slot's clear word, and every CTA adds its counts straight into the output
+ * once it has acquired that word: no combine, and no CTA waits for another at
+ * the end.
+ * Rank 0 clears only once every earlier descriptor of the cluster that
+ * touches the output has finished on every CTA, so a CTA still writing or
+ * reading the same buffer for an earlier descriptor cannot meet the clear:
+ * the output ends as the last descriptor's result, as if the descriptors ran
+ * one by one.  The ones that can still be running are the 7 before this one
+ * (a slot is reused once its descriptor finished).  With outputs apart rank 0
+ * does not wait: waiting for the previous descriptor, whatever it was, made
+ * every histogram wait for the slowest CTA. */
 struct HistSink {
   uint32_t* acc;
-  uint64_t* zero;
+  const lk_cta* cta;
   uint64_t seq;
-  const uint64_t* prev_done;
+  __device__ __forceinline__ uint64_t* clear_word() const { return &cta->dc->hzero[(seq - 1) % LK_BCAST_DEPTH]; }
 };
+
+/* Does descriptor e read or write any byte of [lo, hi)?  (A batch or the
+ * serving queue may.) */
+__device__ __forceinline__ bool touches(const lk_slot& e, uint64_t lo, uint64_t hi) {
+  uint64_t b0 = 0, b1 = 0, bo = 0;
+  switch (e.cmd - LK_CMD_WORK) {
+    case LK_OP_NOP: return false;
+    case LK_OP_ADD_I32: b0 = b1 = bo = 4 * e.n; break;
+    case LK_OP_COPY_I32: b0 = bo = 4 * e.n; break;
+    case LK_OP_HIST_U8: b0 = e.n; bo = 1024; break;
+    case LK_OP_SUM_F32: b0 = 4 * e.n; bo = 4; break;
+    case LK_OP_GEMM64_F32: b0 = b1 = bo = 16384 * e.n; break;
+    case LK_OP_COMBINE_SUM: b0 = 16 * e.n; bo = 4; break;
+    case LK_OP_COMBINE_HIST: b0 = 1024 * e.n; bo = 1024; break;
+    case LK_OP_SPIN: bo = 4 * LK_MAX_CTAS; break;
+    default: return true;
+  }
+  return (e.in0 < hi && e.in0 + b0 > lo) || (e.in1 < hi && e.in1 + b1 > lo) || (e.out < hi && e.out + bo > lo);
+}
+
+/* Rank 0, the whole CTA: wait for the earlier descriptors that touch the
+ * output of descriptor `seq` (one lane of warp 0 each); false, on every
+ * thread, if one did not finish by `deadline`. */
+__device__ __noinline__ bool hist_may_clear(const lk_cta* cta, uint64_t seq, uint64_t deadline) {
+  __shared__ int s_clear;
+  if (threadIdx.x < 32) {
+    const uint64_t k = seq - 1, back = threadIdx.x + 1, out = cta->taken[k % LK_BCAST_DEPTH].out;
+    bool ok = true;
+    if (back < LK_BCAST_DEPTH && back <= k) {
+      const uint32_t i = (uint32_t)((k - back) % LK_BCAST_DEPTH);
+      if (touches(cta->taken[i], out, out + 1024))
+        for (uint32_t it = 0; ld_acquire_gpu(&cta->dc->slot_done[i]) < k - back + 1; ++it)
+          if ((it & 63u) == 63u && gtime() > deadline) {
+            ok = false;
+            break;
+          }
+    }
+    ok = __all_sync(0xffffffffu, ok);
+    if (threadIdx.x == 0) s_clear = ok;
+  }
+  __syncthreads();
+  return s_clear != 0;
+}
 
 /* Thread 0 waits for rank 0's cleared output (with a sink that has one),
  * then the whole CTA synchronises; false, on every thread, if the word did
@@ -665,8 +722,8 @@ __device__ __forceinline__ bool hist_out_ready(const HistSink& sink, uint64_t de
   __shared__ int s_ready;
   if (threadIdx.x == 0) {
     int ready = 1;
-    if (sink.zero)
-      for (uint32_t it = 0; ld_acquire_gpu(sink.zero) < sink.seq; ++it)
+    if (sink.cta)
+      for (uint32_t it = 0; ld_acquire_gpu(sink.clear_word()) < sink.seq; ++it)
         if ((it & 63u) == 63u && gtime() > deadline) {
           ready = 0;
           break;
@@ -691,18 +748,15 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
   const uint4* in = reinterpret_cast<const uint4*>(d.in0);
   bool ok = true;
   const uint64_t total = end - beg;
-  uint32_t* acc = sink.zero ? reinterpret_cast<uint32_t*>(d.out) : sink.acc;
-  /* rank 0 of a sink with a clear word: the counts' targets start at zero;
+  uint32_t* acc = sink.cta ? reinterpret_cast<uint32_t*>(d.out) : sink.acc;
+  /* rank 0 of a cluster: the counts' targets start at zero;
    * the others add once they see it */
   auto clear_out = [&]() -> bool {
-    if (!sink.zero || r != 0) return true;
-    if (sink.prev_done && !hist_out_ready(HistSink{nullptr, const_cast<uint64_t*>(sink.prev_done), sink.seq - 1,
-                                                   nullptr},
-                                          pace.deadline))
-      return false;
+    if (!sink.cta || r != 0) return true;
+    if (!hist_may_clear(sink.cta, sink.seq, pace.deadline)) return false;
     for (uint32_t v = threadIdx.x; v < 256; v += T) acc[v] = 0;
     __syncthreads();
-    if (threadIdx.x == 0) st_release_gpu(sink.zero, sink.seq);
+    if (threadIdx.x == 0) st_release_gpu(sink.clear_word(), sink.seq);
     return true;
   };
   if (total * 16 < LK_HIST_SMALL_BYTES) {

@@ -106,6 +106,15 @@ __device__ __forceinline__ void red_relaxed_gpu_add_s32(int32_t* p, int32_t v) {
 }
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
+/* Named CTA barriers (id 1..15; 0 is __syncthreads): `threads` arrivals open
+ * one; bar_sync waits for it, bar_arrive only counts in.  Whole warps only. */
+__device__ __forceinline__ void bar_sync(uint32_t id, uint32_t threads) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t threads) {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
 /* Exponential back-off between polls.  base == 0 spins without sleeping. */
 struct Backoff {
   uint32_t ns, cap;

@@ -429,6 +429,24 @@ __device__ __noinline__ int serve_take(const lk_kargs& a, uint32_t qlog2, lk_qun
   return 0;
 }
 
+/* Execution-log record of descriptor j (0-based) of this CTA. */
+__device__ __forceinline__ void log_record(const lk_kargs& a, const lk_cta* cta, uint64_t j, uint64_t t_done) {
+  if (!a.log) return;
+  const lk_slot& d = cta->taken[j % LK_BCAST_DEPTH];
+  lk_exec_rec* rec = a.log + (size_t)blockIdx.x * a.log_cap + (j % a.log_cap);
+  rec->seq = d.seq;
+  rec->cluster = (uint32_t)cta->cl;
+  rec->rank = (uint32_t)cta->rank;
+  rec->smid = smid();
+  rec->op = d.cmd - LK_CMD_WORK;
+  rec->order = j;
+  rec->t_pick_ns = cta->t_pick[j & 1u];
+  rec->t_start_ns = cta->t_start[j & 1u];
+  rec->t_end_ns = cta->t_end;
+  rec->t_done_ns = t_done;
+  a.log_count[blockIdx.x] = j + 1;
+}
+
 /* Work units, claimed one at a time by each CTA of the cluster, for two
  * descriptors (one loop, so the bodies are inlined once for both):
  *   LK_OP_BATCH (lk_submit_batch): units from the batch's table in pinned
@@ -557,7 +575,7 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
       ok = body_sum<P, (MAXT <= 256 && P == 1)>(it, (int)part, (int)parts, dsm, bars, phase, deadline, red, pout);
     } else if (op == LK_OP_HIST_U8) {
       ok = body_hist<P, (MAXT <= 256)>(it, (int)part, (int)parts, dsm, bars, phase, deadline,
-                        HistSink{parts > 1 ? s_pbins : my_hist, nullptr, 0, nullptr});
+                        HistSink{parts > 1 ? s_pbins : my_hist, nullptr, 0});
     } else {
       ok = run_body<MAXT, P>(it, (int)part, (int)parts, dsm, bars, phase, red, nullptr, HistSink{}, rate, gate,
                              (a.flags & LK_KFLAG_GEMM_FFMA) == 0) == 0;
@@ -576,7 +594,7 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
     __syncthreads();
     if (s_lastp) {
       if (op == LK_OP_SUM_F32) {
-        if (parts > 1) combine_sum(it, s_psum, (int)parts);
+        if (parts > 1) combine_sum(it, s_psum, (int)parts, threadIdx.x);
         else if (threadIdx.x == 0) *reinterpret_cast<float*>(it.out) = s_part_sum;
       } else if (op == LK_OP_HIST_U8) {
         combine_hist(it, parts > 1 ? s_pbins : my_hist);
@@ -597,15 +615,84 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
   }
 }
 
+/* run_units, out of line in the 1,024-thread kernels: inlined, it shares the
+ * dispatch loop's 64 registers. */
 template <int MAXT, int P>
+__device__ __noinline__ uint32_t call_units(const lk_kargs& a, const lk_slot& d, int c, int r, unsigned char* dsm,
+                                            uint64_t* bars, uint32_t phase, float* red) {
+  const int err = run_units<MAXT, P>(a, d, c, r, dsm, bars, phase, red);
+  return phase | (uint32_t)err << 16;
+}
+template <int MAXT, int P>
+__device__ __forceinline__ int do_units(const lk_kargs& a, const lk_slot& d, int c, int r, unsigned char* dsm,
+                                        uint64_t* bars, uint32_t& phase, float* red) {
+  if constexpr (MAXT > 512) {
+    const uint32_t ret = call_units<MAXT, P>(a, d, c, r, dsm, bars, phase, red);
+    phase = ret & 0xffffu;
+    return (int)(ret >> 16);
+  } else {
+    return run_units<MAXT, P>(a, d, c, r, dsm, bars, phase, red);
+  }
+}
+
+/* Finite mode: warp 1 finishes descriptor j (0-based) -- arrives on the slot,
+ * combines a sum if this CTA arrived last, frees the slot, writes the log
+ * record -- while thread 0 takes the next descriptor and the other warps start
+ * on it; it joins that body at its first CTA barrier.  No completion word is
+ * published: the host waits for the kernel, not for descriptors.  Measured
+ * (152 CTAs, back-to-back NOPs): 3.8 us each with thread 0 doing all of it,
+ * fence and host store included, before the next probe; 3.1 us with warp 1
+ * doing it beside the probe; 2.4 us without the fence and store.  A CTA's gap
+ * between two bodies: 4.25 -> 1.43 us.
+ * Live contexts keep it in line (below): there the completion word is what
+ * the host waits for, and thread 0's probes of the host ring in flight beside
+ * the system-scope fence slowed both (closed-loop adds 4.9 -> 6.2 us).
+ * Out of line: it runs beside the bodies and must not cost them registers.
+ * The whole warp calls it, after the CTA barrier that ends the body. */
+__device__ __noinline__ void finish_finite(const lk_kargs& a, const lk_cta* cta, uint64_t j) {
+  const uint32_t lane = threadIdx.x & 31u, slot = (uint32_t)(j % LK_BCAST_DEPTH);
+  const lk_slot& d = cta->taken[slot];   /* rewritten by descriptor j + 8 */
+  lk_dcluster* dc = cta->dc;
+  const int S = cta->size;
+  int last = S == 1;
+  if (lane == 0 && !last) last = atom_add_acq_rel_gpu(&dc->arrive[slot].count, 1u) == (uint32_t)(S - 1);
+  last = __shfl_sync(0xffffffffu, last, 0);
+  uint64_t t_done = 0;
+  if (last) {
+    if (d.cmd == LK_CMD_WORK + LK_OP_SUM_F32) {
+      combine_sum(d, dc->partial[slot], S, lane);
+      __syncwarp();
+    }
+    if (lane == 0) {
+      if (S > 1) dc->arrive[slot].count = 0;
+      /* the arrivals (acquire-release) order every CTA's reads of the slot and
+       * its partials before this release */
+      st_release_gpu(&dc->slot_done[slot], j + 1);
+      t_done = gtime();
+    }
+  }
+  if (lane == 0) log_record(a, cta, j, t_done);
+  __syncwarp();
+}
+
+/* How the bodies see a descriptor: a copy in registers, or (1,024 threads, 64
+ * registers each) the one in shared memory. */
+template <bool IN_PLACE>
+struct SlotArg { typedef const lk_slot type; };
+template <>
+struct SlotArg<true> { typedef const lk_slot& type; };
+
+/* FINITE: 1 in the kernel that only runs finite contexts, 0 in those that only
+ * run live ones, or finite ones without the overlap (512 and 1,024 threads have
+ * no registers to spare for it), 2 where both run (two CTAs per SM). */
+template <int MAXT, int P, int FINITE>
 __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
   extern __shared__ __align__(128) unsigned char dsm[];
-  __shared__ __align__(64) lk_slot s_desc;
-  __shared__ int32_t s_cl, s_rank, s_size, s_exit, s_err;
-  __shared__ volatile int s_found;     /* rank 0: a warp saw every rank's flag (mailbox mode) */
+  __shared__ lk_cta s_cta;
+  __shared__ int32_t s_exit, s_err;
   __shared__ int32_t s_last;           /* this CTA arrived last on the descriptor's slot */
+  __shared__ volatile int s_found;     /* rank 0: a warp saw every rank's flag (mailbox mode) */
   __shared__ uint64_t s_slot_seen;     /* the slot's completion word, read while probing */
-  __shared__ uint64_t s_tpick, s_tstart; /* thread 0's stamps, for the execution log */
   __shared__ float s_red[32];
   __shared__ __align__(8) uint64_t s_bars[LK_ALL_BARS];
   const uint32_t tid = threadIdx.x;
@@ -679,9 +766,11 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
         rk = pos - a.cl_start[c];
       }
     }
-    s_cl = c;
-    s_rank = rk;
-    s_size = c >= 0 ? a.cl_start[c + 1] - a.cl_start[c] : 0;
+    s_cta.cl = c;
+    s_cta.rank = rk;
+    s_cta.size = c >= 0 ? a.cl_start[c + 1] - a.cl_start[c] : 0;
+    s_cta.dc = a.dcl + (c >= 0 ? c : 0);
+    s_cta.done = a.rdone + (c >= 0 ? a.rd_off[c] + rk : 0);
     lk_cta_info* inf = a.info + blockIdx.x;
     st_relaxed_sys32(&inf->cluster, c);
     st_relaxed_sys32(&inf->rank, rk);
@@ -697,25 +786,27 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
     red_release_sys_add(&a.ctrl->booted, 1u);
   }
   __syncthreads();
-  if (s_cl < 0 || s_err) return;
+  if (s_cta.cl < 0 || s_err) return;
 
-  const int c = s_cl, r = s_rank, S = s_size;
+  const int c = s_cta.cl, r = s_cta.rank, S = s_cta.size;
   const bool master = (r == 0);
   const bool relay = (a.flags & LK_KFLAG_DIRECT) == 0;
   const bool mailbox = (a.flags & LK_KFLAG_MAILBOX) != 0;   /* implies relay */
   lk_dcluster* dc = a.dcl + c;
   const lk_wire* ring = a.ring + (size_t)c * (a.ring_mask + 1);
-  uint64_t* my_done = a.rdone + a.rd_off[c] + r;   /* this CTA's host-visible completion word */
   uint32_t phase = 0;
   int final_err = 0;
   uint64_t known_done = 0;   /* mailbox master: descriptors it completed */
 
+  const uint32_t warp = tid >> 5;
+  const bool overlap = FINITE == 1 || (FINITE == 2 && (a.flags & LK_KFLAG_FINITE) != 0);   /* implies ring mode */
+
   for (uint64_t k = 0;; ++k) {
     const uint32_t slot = (uint32_t)(k % LK_BCAST_DEPTH);
+    lk_slot& dsc = s_cta.taken[slot];   /* written in place: no copy through local memory */
     /* ---- descriptor k+1: from the ring, or from the master's relay ------ */
     if (tid == 0) {
       int err = 0;
-      lk_slot& dsc = s_desc;   /* written in place: no copy through local memory */
       const lk_wire* w = ring + (k & a.ring_mask);
       const uint64_t tag = lk_lap_tag(k, a.ring_log2);
       /* slot k mod D (relay copy, partials, histogram-clear word, arrival
@@ -770,34 +861,47 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       } else {
         s_exit = (dsc.cmd == LK_CMD_EXIT);
       }
-      s_err = 0;
       s_found = 0;
       s_last = 0;
-      s_tpick = t_pick;
-      s_tstart = gtime();
+      s_cta.t_pick[k & 1u] = t_pick;
+      s_cta.t_start[k & 1u] = gtime();
     }
-    __syncthreads();
+    if (overlap) {
+      __syncwarp();
+      /* two barriers, so that no warp waits for warp 1 here: the others meet
+       * thread 0 at the first (warp 1 only arrives, and then finishes the
+       * previous descriptor), and warp 1 meets them at the second (they only
+       * arrive) */
+      if (warp == 1) {
+        bar_arrive(1, blockDim.x);
+        if (k > 0) finish_finite(a, &s_cta, k - 1);
+        bar_sync(2, blockDim.x);
+      } else {
+        bar_sync(1, blockDim.x);
+        bar_arrive(2, blockDim.x);
+      }
+    } else {
+      __syncthreads();
+    }
     if (s_exit) break;
 
     /* ---- run this CTA's share ------------------------------------------ */
-    const lk_slot d = s_desc;
+    typename SlotArg<(MAXT > 512)>::type d = dsc;
     const uint32_t op = d.cmd - LK_CMD_WORK;
     const int berr = (op == LK_OP_BATCH || op == LK_OP_SERVE)
-                         ? run_units<MAXT, P>(a, d, c, r, dsm, s_bars, phase, s_red)
+                         ? do_units<MAXT, P>(a, d, c, r, dsm, s_bars, phase, s_red)
                          : run_body<MAXT, P>(d, r, S, dsm, s_bars, phase, s_red, &dc->partial[slot][r],
-                                             HistSink{nullptr, &dc->hzero[slot], d.seq,
-                                                      k > 0 && !mailbox ? &dc->slot_done[(k - 1) % LK_BCAST_DEPTH]
-                                                                        : nullptr},
+                                             HistSink{nullptr, &s_cta, d.seq},
                                              cta_rate(d.aux, S), (d.flags & LK_DFLAG_YIELD) ? a.crit_active : nullptr,
                                              (a.flags & LK_KFLAG_GEMM_FFMA) == 0);
-    if (berr && tid == 0) s_err = berr;
+    if (berr) s_err = berr;   /* 0 until then */
     __syncthreads();
 
-    uint64_t t_end = 0, t_done = 0;
-    if (tid == 0) t_end = gtime();
     if (mailbox) {
       /* ---- finish, one-deep mailbox: rank 0 gathers every rank's flag,
        * combines a sum, and answers THREAD_FINISHED ---------------------- */
+      uint64_t t_done = 0;
+      if (tid == 0) s_cta.t_end = gtime();
       if (tid == 0 && S > 1) st_release_gpu(&dc->flag[r], k + 1);   /* orders this CTA's writes (after the barrier) */
       if (master) {
         if (S > 1) {
@@ -806,7 +910,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
         }
         __syncthreads();
         if (!s_err) {
-          if (op == LK_OP_SUM_F32) combine_sum(d, dc->partial[slot], S);
+          if (op == LK_OP_SUM_F32 && warp == 0) combine_sum(d, dc->partial[slot], S, tid);
           __syncthreads();
           if (tid == 0) {
             if (op == LK_OP_BATCH) a.bcl[c].ticket = 0;   /* every rank has left the claim loop */
@@ -821,6 +925,9 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
           }
         }
       }
+      if (tid == 0) log_record(a, &s_cta, k, t_done);
+    } else if (overlap) {
+      if (tid == 32) s_cta.t_end = gtime();   /* warp 1 finishes it beside the next one */
     } else {
       /* ---- finish, ring modes: every CTA publishes its own completion
        * word (the paper's per-SM from_GPU mailbox); the host takes the
@@ -832,13 +939,15 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
        * combine).  Other ops -- a histogram too: every CTA adds its counts
        * into the output itself -- arrive after publishing, off the host's
        * path; their arrivals only pick the CTA that frees the slot. */
+      uint64_t t_done = 0;
+      if (tid == 0) s_cta.t_end = gtime();
       const bool comb = op == LK_OP_SUM_F32 || op == LK_OP_BATCH;
       if (comb) {
         if (tid == 0 && !s_err)
           s_last = S == 1 || atom_add_acq_rel_gpu(&dc->arrive[slot].count, 1u) == (uint32_t)(S - 1);
         __syncthreads();
         if (s_last) {   /* CTA-uniform after the barrier */
-          if (op == LK_OP_SUM_F32) combine_sum(d, dc->partial[slot], S);
+          if (op == LK_OP_SUM_F32) combine_sum(d, dc->partial[slot], S, tid);
           __syncthreads();   /* the combine's writes before thread 0's fence */
         }
       }
@@ -847,7 +956,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
          * ran it; the barrier above orders the other threads' writes) before
          * the host-visible word */
         fence_acq_rel_sys();
-        st_relaxed_sys(my_done, k + 1);
+        st_relaxed_sys(s_cta.done, k + 1);
         if (!comb) s_last = S == 1 || atom_add_acq_rel_gpu(&dc->arrive[slot].count, 1u) == (uint32_t)(S - 1);
         if (s_last) {
           /* every CTA has arrived: free the slot (the arrivals, acquire-
@@ -860,22 +969,9 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
           t_done = gtime();
         }
       }
+      if (tid == 0) log_record(a, &s_cta, k, t_done);
     }
-    if (tid == 0 && a.log) {
-      lk_exec_rec* rec = a.log + (size_t)blockIdx.x * a.log_cap + (k % a.log_cap);
-      rec->seq = d.seq;
-      rec->cluster = (uint32_t)c;
-      rec->rank = (uint32_t)r;
-      rec->smid = smid();
-      rec->op = op;
-      rec->order = k;
-      rec->t_pick_ns = s_tpick;
-      rec->t_start_ns = s_tstart;
-      rec->t_end_ns = t_end;
-      rec->t_done_ns = t_done;
-      a.log_count[blockIdx.x] = k + 1;
-    }
-    __syncthreads();
+    if (!overlap) __syncthreads();
     if (s_err) {
       if (tid == 0) {
         set_error(a, c, (uint32_t)s_err);
@@ -885,6 +981,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       break;
     }
   }
+  __syncthreads();   /* warp 1's completion word before thread 0 reports the exit */
   if (tid == 0) {
     if (master && mailbox) {
       /* completions the host has not consumed through FINISHED yet stay
@@ -900,13 +997,13 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
 /* The persistent kernel (live contexts: lk_init). */
 template <int MAXT, int P>
 __global__ void __launch_bounds__(MAXT, P) lk_persistent(const lk_kargs a) {
-  persistent_main<MAXT, P>(a);
+  persistent_main<MAXT, P, P == 2 ? 2 : 0>(a);
 }
 
 /* The same kernel under another name for finite mode (lk_run_finite, 256
  * threads, one CTA per SM), so that a profiler can select its launches
  * apart from live contexts, which wait on the host and cannot be replayed. */
-__global__ void __launch_bounds__(256, 1) lk_finite(const lk_kargs a) { persistent_main<256, 1>(a); }
+__global__ void __launch_bounds__(256, 1) lk_finite(const lk_kargs a) { persistent_main<256, 1, 1>(a); }
 
 /* ---- ordinary-launch baseline: the same bodies, one launch per item ------ */
 struct lk_scratch {
@@ -932,7 +1029,7 @@ __global__ void __launch_bounds__(MAXT) lk_ordinary(const lk_slot d, lk_scratch*
   }
   __syncthreads();
   uint32_t phase = 0;
-  run_body<MAXT, 1>(d, r, S, dsm, s_bars, phase, s_red, &sc->partial[r], HistSink{sc->hist, nullptr, 0, nullptr}, 0, nullptr);
+  run_body<MAXT, 1>(d, r, S, dsm, s_bars, phase, s_red, &sc->partial[r], HistSink{sc->hist, nullptr, 0}, 0, nullptr);
   if (op != LK_OP_SUM_F32 && op != LK_OP_HIST_U8) return;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -941,7 +1038,7 @@ __global__ void __launch_bounds__(MAXT) lk_ordinary(const lk_slot d, lk_scratch*
   }
   __syncthreads();
   if (s_last) {
-    if (op == LK_OP_SUM_F32) combine_sum(d, sc->partial, S);
+    if (op == LK_OP_SUM_F32) combine_sum(d, sc->partial, S, threadIdx.x);
     else combine_hist(d, sc->hist);
     __syncthreads();
     if (threadIdx.x == 0) sc->counter = 0;

@@ -406,7 +406,13 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   a.flags = ((p->flags & LK_INIT_DIRECT) ? LK_KFLAG_DIRECT : 0u) | (ctx->mailbox ? LK_KFLAG_MAILBOX : 0u);
   a.ctas_per_sm = ctx->per_sm;
   if (p->flags & LK_INIT_GEMM_FFMA) a.flags |= LK_KFLAG_GEMM_FFMA;
-  if (!live) a.flags |= LK_KFLAG_FINITE;
+  /* finite mode's ring lies in device memory, where any number of readers is
+   * cheap: every CTA takes its descriptors itself, up to 8 ahead of the
+   * slowest, beside finishing the one before (no relay through rank 0).  The
+   * 512- and 1,024-thread kernels finish first (finish_finite): there every
+   * CTA's own fence costs more than the relay (1,024 threads: 5.8 us a NOP
+   * against 4.8) */
+  if (!live) a.flags |= LK_KFLAG_FINITE | (ctx->T <= 256 ? LK_KFLAG_DIRECT : 0u);
   a.backoff_base_ns = p->backoff_base_ns;
   a.backoff_cap_ns = p->backoff_cap_ns ? p->backoff_cap_ns : 256;
   a.lease_ns = p->idle_lease_ns ? p->idle_lease_ns : 10000000000ull;

@@ -4,7 +4,11 @@ small-share cut, one granule more or less than a stage or a ring, every number
 of rings before and after the table (the block size sets it), and tile counts
 around the wrap of the stages and buffers.  The bounds-checking build runs
 them, so every region is checked too.  Histograms are exact; GEMM elements
-stay within 1e-4 sum|a b| of binary64."""
+stay within 1e-4 sum|a b| of binary64.
+
+Also the histogram's clearing of its output, which waits only for earlier
+descriptors that touch it: other writers of the same buffer, neighbours that
+end where it starts, and more than a relay ring of them in flight."""
 import numpy as np
 import pytest
 
@@ -54,3 +58,34 @@ def test_gemm_tile_counts(torch_ready, oracle_lib, S):
     for A, B, _, _, dC in cases:
         assert gemm_ok(host(dC), A, B, oracle_lib), A.shape
     assert lk.lk_bounds_violations() == (0, 0)
+
+
+@pytest.mark.parametrize("finite", [False, True])
+@pytest.mark.parametrize("per_sm", [1, 2])
+def test_hist_clear_after_earlier_writers(torch_ready, oracle_lib, finite, per_sm):
+    torch = torch_ready
+    S, rounds = 9, 12
+    xs = [synth.bytes_uniform(33, i, 200_000 + 977 * i) for i in range(rounds)]
+    a = synth.int32_uniform(33, 99, 1024, -(1 << 20), 1 << 20)
+    dxs, da = [to_dev(x) for x in xs], to_dev(a)
+    buf = torch.zeros(1024, dtype=torch.int32, device="cuda")       # histograms go to words 256..511
+    apart = torch.full((rounds, 256), -1, dtype=torch.int32, device="cuda")
+    rows = []
+    for i in range(rounds):
+        rows.append((lk.LK_OP_ADD_I32, 512, (da, da), buf.data_ptr()))                    # covers the output
+        rows.append((lk.LK_OP_HIST_U8, xs[i].size, (dxs[i],), buf.data_ptr() + 1024))
+        rows.append((lk.LK_OP_COPY_I32, 256, (da,), buf.data_ptr()))                      # ends where it starts
+        rows.append((lk.LK_OP_HIST_U8, xs[i].size, (dxs[i],), apart[i]))
+    torch.cuda.current_stream().synchronize()
+    if finite:
+        lk.lk_run_finite([S], [(op, n) for op, n, _, _ in rows], [0] * len(rows), in0=[ins[0] for _, _, ins, _ in rows],
+                         in1=[ins[1] if len(ins) > 1 else None for _, _, ins, _ in rows], out=[o for *_, o in rows],
+                         ctas_per_sm=per_sm)
+    else:
+        with lk.lk_init([S], idle_lease_ns=5_000_000_000, ctas_per_sm=per_sm) as c:
+            hs = [lk.lk_submit(c, 0, op, n, ins, out) for op, n, ins, out in rows]
+            for h in hs:
+                assert lk.lk_wait(c, h) == lk.LK_OK, lk.lk_device_error(c)
+    assert np.array_equal(host(buf)[256:512].astype(np.int64), oracle_lib.hist_u8(xs[-1]))
+    for i in range(rounds):
+        assert np.array_equal(host(apart)[i].astype(np.int64), oracle_lib.hist_u8(xs[i])), i
