@@ -25,9 +25,9 @@ typedef struct {
 typedef struct lkb_launch lkb_launch;
 
 int  lkb_props_get(int device, lkb_props* out);                      /* LK_OK / LK_EDEVICE */
-int  lkb_alloc_mapped(int device, size_t bytes, void** host, void** dev); /* zeroed */
+int  lkb_alloc_mapped(int device, size_t bytes, size_t zero_bytes, void** host, void** dev); /* the first zero_bytes zeroed */
 void lkb_free_mapped(void* host);
-int  lkb_alloc_device(int device, size_t bytes, void** dev);           /* zeroed */
+int  lkb_alloc_device(int device, size_t bytes, void** dev);           /* not zeroed */
 void lkb_free_device(void* dev);
 int  lkb_zero_device(int device, void* dev, size_t bytes);           /* copy engine, not SMs */
 int  lkb_copy_h2d(int device, void* dst, const void* src, size_t bytes);
@@ -37,8 +37,12 @@ int  lkb_stream_create(int device, void** stream);
 int  lkb_memcpy_async(void* stream, void* dst, const void* src, size_t bytes, int host_to_device);
 int  lkb_stream_sync(void* stream);
 void lkb_stream_destroy(void* stream);
-/* Launch the persistent kernel: a->grid CTAs of `threads` threads. */
-int  lkb_launch_kernel(int device, const lk_kargs* a, int threads, lkb_launch** out);
+/* Launch the persistent kernel: a->grid CTAs of `threads` threads.  Before it
+ * runs, `head_bytes` at head_src (pinned host memory that stays as it is until
+ * the kernel has booted) are copied to head_dst on its stream, without a wait;
+ * at boot it clears a->zero_base[0 .. zero_bytes). */
+int  lkb_launch_kernel(int device, const lk_kargs* a, int threads, void* head_dst, const void* head_src,
+                       size_t head_bytes, lkb_launch** out);
 /* 1 = kernel returned, 0 = still running, < 0 = LK_EDEVICE. */
 int  lkb_finished(lkb_launch* l);
 /* Elapsed CUDA-event time of the launch in ms (after it finished), or -1. */

@@ -67,10 +67,11 @@ int lkb_props_get(int device, lkb_props* out) {
   return LK_OK;
 }
 
-int lkb_alloc_mapped(int, size_t bytes, void** host, void** dev) {
+int lkb_alloc_mapped(int, size_t bytes, size_t zero_bytes, void** host, void** dev) {
   void* p = aligned_alloc(4096, (bytes + 4095) / 4096 * 4096);
   if (!p) return LK_ENOMEM;
-  memset(p, 0, bytes);
+  memset(p, 0xee, bytes);   /* recycled memory holds anything */
+  memset(p, 0, zero_bytes);
   *host = *dev = p;
   return LK_OK;
 }
@@ -78,6 +79,7 @@ void lkb_free_mapped(void* host) { free(host); }
 int lkb_alloc_device(int, size_t bytes, void** dev) {
   void* p = aligned_alloc(4096, (bytes + 4095) / 4096 * 4096);
   if (!p) return LK_ENOMEM;
+  memset(p, 0xee, bytes);
   *dev = p;
   return LK_OK;
 }
@@ -183,7 +185,7 @@ static void cluster_loop(lk_kargs a, int c, std::vector<int> ctas, std::vector<i
   };
   for (uint64_t k = 0;; ++k) {
     uint32_t cmd = 0;
-    uint64_t in0 = 0;
+    uint64_t in0 = 0, out = 0, n = 0;
     if (mailbox) {
       /* the one-deep mailbox: acknowledge the host's re-arm, then take work */
       lk_mbox* mb = a.mbox + c;
@@ -215,9 +217,12 @@ static void cluster_loop(lk_kargs a, int c, std::vector<int> ctas, std::vector<i
       lk_wire_decode(w, k + 1, &dsc);
       cmd = dsc.cmd;
       in0 = dsc.in0;
+      out = dsc.out;
+      n = dsc.n;
     }
     if (cmd == LK_CMD_EXIT) break;
     if (k >= fail_after) { err = fail_code; break; }
+    if (cmd == LK_CMD_WORK + LK_OP_ZERO) memset((void*)out, 0, n);
     if (cmd == LK_CMD_WORK + LK_OP_SERVE) {
       err = serve(reinterpret_cast<lk_qstate*>(in0));
       if (err) break;
@@ -258,9 +263,12 @@ static void cluster_loop(lk_kargs a, int c, std::vector<int> ctas, std::vector<i
   l->alive.fetch_sub(1);
 }
 
-int lkb_launch_kernel(int, const lk_kargs* ap, int threads, lkb_launch** out) {
+int lkb_launch_kernel(int, const lk_kargs* ap, int threads, void* head_dst, const void* head_src, size_t head_bytes,
+                      lkb_launch** out) {
   if (threads < 64) return LK_EDEVICE;
   const lk_kargs a = *ap;
+  memcpy(head_dst, head_src, head_bytes);
+  memset(a.zero_base, 0, a.zero_bytes);
   lkb_launch* l = new lkb_launch();
   l->t0 = now_ns();
   const int sms = fake_sms();

@@ -889,6 +889,15 @@ __device__ __forceinline__ void body_spin(const lk_slot& d, int r, uint32_t* red
   }
 }
 
+/* ---- clearing (lk_serve's queue state) ------------------------------------ */
+__device__ __forceinline__ void body_zero(const lk_slot& d, int r, int S) {
+  uint64_t beg, end;
+  share(d.n >> 4, r, S, beg, end);
+  uint4* o = reinterpret_cast<uint4*>(d.out);
+  for (uint64_t v = beg + threadIdx.x; v < end; v += blockDim.x)
+    if (LK_INB(v < d.n >> 4, LK_OOB_STORE)) o[v] = make_uint4(0, 0, 0, 0);
+}
+
 /* ---- combining chunk results (rank 0 of the cluster alone) ------------- */
 /* out[0] = binary64 sum of n float32 partials, one per 16-byte slot, added
  * lane-strided then by a fixed shuffle tree: the order depends only on n. */

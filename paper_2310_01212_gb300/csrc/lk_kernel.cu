@@ -380,6 +380,7 @@ __device__ __forceinline__ int run_body(const lk_slot& d, int r, int S, unsigned
     case LK_OP_COMBINE_HIST: body_combine_hist(d, r); break;
     case LK_OP_SPIN: body_spin(d, r, reinterpret_cast<uint32_t*>(red)); break;
     case LK_OP_NOP: break;
+    case LK_OP_ZERO: body_zero(d, r, S); break;
     default: return LK_DERR_BADDESC;
   }
 #ifdef LK_DEBUG_BOUNDS
@@ -697,8 +698,17 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
   __shared__ __align__(8) uint64_t s_bars[LK_ALL_BARS];
   const uint32_t tid = threadIdx.x;
 
-  /* ---- boot: read %smid, exchange, join a cluster --------------------- */
+  /* ---- boot: clear the control state, read %smid, exchange, join a
+   * cluster.  The state (45 KB a cluster, live contexts 350 KB and 1 KB a CTA
+   * more) is cleared by all CTAs before the grid barrier below; sent from
+   * pageable host memory it took lk_run_finite 0.1 ms a cluster. */
   __shared__ int32_t s_sm, s_slot, s_pos;
+  {
+    uint4* z = reinterpret_cast<uint4*>(a.zero_base);
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + tid; i < a.zero_bytes / 16u; i += (uint64_t)a.grid * blockDim.x)
+      z[i] = make_uint4(0, 0, 0, 0);
+  }
+  __syncthreads();
   if (tid == 0) {
     s_err = 0;
     s_slot = 0;
@@ -1065,6 +1075,21 @@ __global__ void lk_pingpong_kernel(const uint64_t* ping, uint64_t* pong, int ite
 /* ======================================================================= */
 namespace {
 
+/* Properties of a device (immutable), read once: the query takes longer than
+ * a launch.  nullptr if the device cannot be read. */
+const cudaDeviceProp* dev_props(int device) {
+  static std::mutex mu;
+  static cudaDeviceProp props[64];
+  static bool known[64];
+  if (device < 0 || device >= 64) return nullptr;
+  std::lock_guard<std::mutex> g(mu);
+  if (!known[device]) {
+    if (cudaGetDeviceProperties(&props[device], device) != cudaSuccess) return nullptr;
+    known[device] = true;
+  }
+  return &props[device];
+}
+
 std::once_flag g_preload_once;
 cudaError_t g_preload_err = cudaSuccess;
 
@@ -1192,8 +1217,9 @@ struct lkb_launch {
 };
 
 int lkb_props_get(int device, lkb_props* out) {
-  cudaDeviceProp p;
-  if (cudaGetDeviceProperties(&p, device) != cudaSuccess) return LK_EDEVICE;
+  const cudaDeviceProp* pp = dev_props(device);
+  if (!pp) return LK_EDEVICE;
+  const cudaDeviceProp& p = *pp;
   out->sm_count = p.multiProcessorCount;
   out->smem_per_sm = p.sharedMemPerMultiprocessor;
   out->smem_per_block_optin = p.sharedMemPerBlockOptin;
@@ -1203,11 +1229,11 @@ int lkb_props_get(int device, lkb_props* out) {
   return LK_OK;
 }
 
-int lkb_alloc_mapped(int device, size_t bytes, void** host, void** dev) {
+int lkb_alloc_mapped(int device, size_t bytes, size_t zero_bytes, void** host, void** dev) {
   Block b;
   int rc = take_block(device, bytes, true, &b);
   if (rc != LK_OK) return rc;
-  memset(b.host, 0, bytes);
+  memset(b.host, 0, zero_bytes);
   *host = b.host;
   *dev = b.dev;
   return LK_OK;
@@ -1256,36 +1282,77 @@ void lkb_stream_destroy(void* stream) {
   if (stream) cudaStreamDestroy((cudaStream_t)stream);
 }
 
-int lkb_launch_kernel(int device, const lk_kargs* a, int threads, lkb_launch** out) {
-  *out = nullptr;
-  if (cudaSetDevice(device) != cudaSuccess) return LK_EDEVICE;
-  preload_all();
-  if (g_preload_err != cudaSuccess) return LK_EDEVICE;
-  cudaDeviceProp p;
-  if (cudaGetDeviceProperties(&p, device) != cudaSuccess) return LK_EDEVICE;
-  const int want = a->ctas_per_sm == 2 ? 2 : 1;
-  const void* fn = persistent_fn(threads, want, (a->flags & LK_KFLAG_FINITE) != 0);
-  if (!fn) return LK_EINVAL;
-  /* exactly `want` CTAs per SM: ask for more than 1/(want+1) of the SM's
-   * shared memory (one CTA: more than half; two: more than a third) */
-  size_t dyn = std::max<size_t>(lk::body_smem_bytes(want), p.sharedMemPerMultiprocessor / (want + 1) + 1);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-    return LK_EDEVICE;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, dyn) != cudaSuccess) return LK_EDEVICE;
-  if (per_sm != want || a->grid > want * p.multiProcessorCount) return LK_EDEVICE;
+namespace {
+
+/* Streams and events of finished launches, kept for the next one (a stream and
+ * two events take longer to make than a launch): at most kKeep a device. */
+constexpr size_t kKeep = 4;
+std::mutex g_launch_mu;
+std::vector<lkb_launch*> g_launches;
+
+lkb_launch* take_launch(int device) {
+  {
+    std::lock_guard<std::mutex> g(g_launch_mu);
+    for (size_t i = 0; i < g_launches.size(); ++i)
+      if (g_launches[i]->device == device) {
+        lkb_launch* l = g_launches[i];
+        g_launches.erase(g_launches.begin() + (long)i);
+        return l;
+      }
+  }
   lkb_launch* l = new lkb_launch{device, nullptr, nullptr, nullptr};
   if (cudaStreamCreateWithFlags(&l->s, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreate(&l->e0) != cudaSuccess || cudaEventCreate(&l->e1) != cudaSuccess) {
     lkb_release(l);
-    return LK_EDEVICE;
+    return nullptr;
   }
+  return l;
+}
+
+/* The shared-memory request that fits exactly `want` CTAs of fn on an SM (one
+ * CTA: more than half of it; two: more than a third), with the function set
+ * up for it; checked once per function, block size and device.  0: it does
+ * not fit that way. */
+size_t launch_smem(int device, const cudaDeviceProp& p, const void* fn, int threads, int want) {
+  struct Known { int device; const void* fn; int threads; size_t dyn; };
+  static std::mutex mu;
+  static std::vector<Known> known;   /* at most one entry per kernel, block size and device */
+  std::lock_guard<std::mutex> g(mu);
+  for (const Known& k : known)
+    if (k.device == device && k.fn == fn && k.threads == threads) return k.dyn;
+  const size_t dyn = std::max<size_t>(lk::body_smem_bytes(want), p.sharedMemPerMultiprocessor / (want + 1) + 1);
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return 0;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, dyn) != cudaSuccess || per_sm != want) return 0;
+  known.push_back({device, fn, threads, dyn});
+  return dyn;
+}
+
+}  // namespace
+
+int lkb_launch_kernel(int device, const lk_kargs* a, int threads, void* head_dst, const void* head_src,
+                      size_t head_bytes, lkb_launch** out) {
+  *out = nullptr;
+  if (cudaSetDevice(device) != cudaSuccess) return LK_EDEVICE;
+  preload_all();
+  if (g_preload_err != cudaSuccess) return LK_EDEVICE;
+  const cudaDeviceProp* p = dev_props(device);
+  if (!p) return LK_EDEVICE;
+  const int want = a->ctas_per_sm == 2 ? 2 : 1;
+  const void* fn = persistent_fn(threads, want, (a->flags & LK_KFLAG_FINITE) != 0);
+  if (!fn) return LK_EINVAL;
+  const size_t dyn = launch_smem(device, *p, fn, threads, want);
+  if (!dyn || a->grid > want * p->multiProcessorCount) return LK_EDEVICE;
+  lkb_launch* l = take_launch(device);
+  if (!l) return LK_EDEVICE;
   lk_kargs args = *a;
   void* params[] = {&args};
-  cudaEventRecord(l->e0, l->s);
-  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(a->grid), dim3(threads), params, dyn, l->s);
+  cudaError_t e = cudaMemcpyAsync(head_dst, head_src, head_bytes, cudaMemcpyHostToDevice, l->s);
+  if (e == cudaSuccess) e = cudaEventRecord(l->e0, l->s);
+  if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(fn, dim3(a->grid), dim3(threads), params, dyn, l->s);
   if (e != cudaSuccess) {
     if (getenv("LK_LOG")) fprintf(stderr, "lk: cooperative launch failed: %s\n", cudaGetErrorString(e));
+    cudaStreamSynchronize(l->s);   /* the copy, before its source is given back */
     lkb_release(l);
     return LK_EDEVICE;
   }
@@ -1310,6 +1377,15 @@ float lkb_elapsed_ms(lkb_launch* l) {
 
 void lkb_release(lkb_launch* l) {
   if (!l) return;
+  if (l->s && l->e0 && l->e1 && cudaStreamQuery(l->s) == cudaSuccess) {
+    std::lock_guard<std::mutex> g(g_launch_mu);
+    size_t kept = 0;
+    for (const lkb_launch* k : g_launches) kept += k->device == l->device;
+    if (kept < kKeep) {
+      g_launches.push_back(l);
+      return;
+    }
+  }
   if (l->e0) cudaEventDestroy(l->e0);
   if (l->e1) cudaEventDestroy(l->e1);
   if (l->s) cudaStreamDestroy(l->s);
@@ -1620,7 +1696,7 @@ extern "C" int lk_pingpong(int device, int iters, uint64_t* rtt_ns) {
   if (cudaSetDevice(device) != cudaSuccess) return LK_EDEVICE;
   preload_all();
   void *h = nullptr, *dptr = nullptr;
-  int rc = lkb_alloc_mapped(device, 4096, &h, &dptr);
+  int rc = lkb_alloc_mapped(device, 4096, 4096, &h, &dptr);
   if (rc != LK_OK) return rc;
   uint64_t* ping = (uint64_t*)h;
   uint64_t* pong = (uint64_t*)h + 16;

@@ -213,6 +213,10 @@ typedef struct __attribute__((aligned(64))) {
 
 #define LK_SERVE_MAX_PARTS 1024   /* work units of one request           */
 
+/* lk_serve's own operation, never user-set: clear n bytes (a multiple of 16)
+ * at out, shared by the cluster's CTAs. */
+#define LK_OP_ZERO 11
+
 typedef struct __attribute__((aligned(LK_LINE))) {
   uint32_t done;                  /* parts finished (the last one resets it)  */
   uint8_t pad[LK_LINE - 4];
@@ -264,6 +268,8 @@ typedef struct {
   lk_bcluster* bcl;              /* [C] device: batch tickets and combine state         */
   uint32_t* cta_hist;            /* [total][256] device: single-part histogram bins     */
   int32_t* crit_active;          /* device: critical descriptors running (lk_set_role)  */
+  void* zero_base;               /* device: state the kernel clears at boot (128-byte   */
+  uint64_t zero_bytes;           /* aligned, a multiple of 16 bytes)                    */
   int32_t num_clusters;
   int32_t grid;
   int32_t total;                 /* CTAs that join clusters (= sum of sizes)            */

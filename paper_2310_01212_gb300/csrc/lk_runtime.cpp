@@ -66,7 +66,7 @@ struct lk_ctx {
 
   void* mapped_h = nullptr;
   void* mapped_d = nullptr;
-  lk_wire* ring_h = nullptr;     /* host view of the ring (live mode) */
+  lk_wire* ring_h = nullptr;     /* host view of the ring (finite mode: the copy that is sent) */
   uint32_t R_log2 = 10;
   lk_cword* cword_h = nullptr;
   uint64_t* rdone_h = nullptr;   /* per-CTA completion words (ring modes) */
@@ -75,6 +75,8 @@ struct lk_ctx {
   lk_cta_info* info_h = nullptr;
 
   void* dev_base = nullptr;
+  const char* head_h = nullptr;  /* pinned copy of the first head_bytes of dev_base, sent with the launch */
+  size_t head_bytes = 0;
   lk_kargs args{};
   uint32_t log_cap = 0;
 
@@ -296,8 +298,10 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   if ((p->flags & LK_INIT_DIRECT) && (p->flags & LK_INIT_MAILBOX)) return LK_EINVAL;
   ctx->mailbox = live && (p->flags & LK_INIT_MAILBOX);
 
-  /* host-mapped block: [ring (live only)] cword[C] rdone[..] ctrl info[G] [unit tables, mailboxes,
-   * serving queue (live only)] */
+  /* host-mapped block: [ring (live only)] cword[C] rdone[..] ctrl info[G] [mailboxes, close word (live
+   * only)] head, all cleared here, then [unit tables, serving queue (live only)], which are written before
+   * they are read (lk_submit_batch, serve_queue) and not cleared: they are 0.8 MB a cluster and 4.7 MB,
+   * most of what lk_init used to spend its time on */
   ctx->max_units = live ? (p->max_batch_units ? p->max_batch_units : 8192u) : 0u;
   if (ctx->max_units > (1u << 22)) return LK_EINVAL;
   size_t off_ring = 0;
@@ -313,20 +317,28 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   size_t off_rd = align_up(off_cw + ctx->C * sizeof(lk_cword), LK_LINE);
   size_t off_ctrl = align_up(off_rd + rd_words * sizeof(uint64_t), LK_LINE);
   size_t off_info = align_up(off_ctrl + sizeof(lk_ctrl), LK_LINE);
-  size_t off_units = align_up(off_info + ctx->G * sizeof(lk_cta_info), LK_LINE);
-  size_t units_bytes = (size_t)ctx->C * LK_BATCH_BUFFERS * ctx->max_units * sizeof(lk_unit);
-  size_t off_mbox = align_up(off_units + units_bytes, LK_LINE);
+  size_t off_mbox = align_up(off_info + ctx->G * sizeof(lk_cta_info), LK_LINE);
   size_t mbox_bytes = ctx->mailbox ? ctx->C * sizeof(lk_mbox) : 0;
-  /* the serving queue: unit ring, completion ring, close word (live only) */
+  size_t off_close = align_up(off_mbox + mbox_bytes, LK_LINE);
+  /* the head: what the kernel reads from device memory, sent in one copy with the launch:
+   * [ring (finite only)] cl_start rd_off pin_smid boot_count */
+  size_t d_start = live ? 0 : align_up(ring_bytes, LK_LINE);
+  size_t d_rdoff = align_up(d_start + (ctx->C + 1) * sizeof(int32_t), LK_LINE);
+  size_t d_pin = align_up(d_rdoff + ctx->C * sizeof(int32_t), LK_LINE);
+  size_t d_bcnt = align_up(d_pin + (p->smids ? ctx->total : 0) * sizeof(int32_t), LK_LINE);
+  ctx->head_bytes = align_up(d_bcnt + sizeof(uint32_t), LK_LINE);
+  size_t off_head = align_up(off_close + LK_LINE, LK_LINE);
+  size_t off_units = align_up(off_head + ctx->head_bytes, LK_LINE);
+  size_t units_bytes = (size_t)ctx->C * LK_BATCH_BUFFERS * ctx->max_units * sizeof(lk_unit);
+  /* the serving queue: unit ring, completion ring (live only) */
   ctx->qn = live ? (p->serve_units ? p->serve_units : 65536u) : 0u;
   if (live && (ctx->qn < 256 || ctx->qn > (1u << 22) || (ctx->qn & (ctx->qn - 1)))) return LK_EINVAL;
   ctx->qlog2 = 0;
   while (ctx->qn && (1u << ctx->qlog2) < ctx->qn) ctx->qlog2++;
-  size_t off_q = align_up(off_mbox + mbox_bytes, LK_LINE);
+  size_t off_q = align_up(off_units + units_bytes, LK_LINE);
   size_t off_cq = align_up(off_q + (size_t)ctx->qn * sizeof(lk_qunit), LK_LINE);
-  size_t off_close = align_up(off_cq + (size_t)ctx->qn * sizeof(uint64_t), LK_LINE);
-  size_t mapped_bytes = align_up(off_close + (ctx->qn ? LK_LINE : 0), 4096);
-  rc = lkb_alloc_mapped(ctx->device, mapped_bytes, &ctx->mapped_h, &ctx->mapped_d);
+  size_t mapped_bytes = align_up(off_cq + (size_t)ctx->qn * sizeof(uint64_t), 4096);
+  rc = lkb_alloc_mapped(ctx->device, mapped_bytes, off_units, &ctx->mapped_h, &ctx->mapped_d);
   if (rc != LK_OK) return rc;
   char* mh = (char*)ctx->mapped_h;
   char* md = (char*)ctx->mapped_d;
@@ -351,32 +363,26 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
     for (int c = 0; c < ctx->C; ++c) ctx->mbox_h[c].to_gpu = LK_CMD_NOP;   /* idle */
   }
 
-  /* device block: [ring (finite only)] dcl[C] cl_start rd_off pin_smid boot_smid boot_count crit_active
-   * log_count bcl chist log */
+  /* device block: head; then the control state that starts at zero, which the kernel's CTAs clear at
+   * boot: dcl[C] crit_active log_count [bcl chist (live only)]; then what needs no clearing:
+   * boot_smid log */
   size_t d_ring = 0;
-  size_t d_dcl = live ? 0 : align_up(ring_bytes, LK_LINE);
-  size_t d_start = align_up(d_dcl + ctx->C * sizeof(lk_dcluster), LK_LINE);
-  size_t d_rdoff = align_up(d_start + (ctx->C + 1) * sizeof(int32_t), LK_LINE);
-  size_t d_pin = align_up(d_rdoff + ctx->C * sizeof(int32_t), LK_LINE);
-  size_t d_bsm = align_up(d_pin + (p->smids ? ctx->total : 0) * sizeof(int32_t), LK_LINE);
-  size_t d_bcnt = align_up(d_bsm + ctx->G * sizeof(int32_t), LK_LINE);
-  size_t d_crit = align_up(d_bcnt + sizeof(uint32_t), LK_LINE);
+  size_t d_dcl = ctx->head_bytes;
+  size_t d_crit = align_up(d_dcl + ctx->C * sizeof(lk_dcluster), LK_LINE);
   size_t d_lcnt = align_up(d_crit + sizeof(int32_t), LK_LINE);
   size_t d_bcl = align_up(d_lcnt + ctx->G * sizeof(uint64_t), LK_LINE);
-  size_t d_chist = align_up(d_bcl + ctx->C * sizeof(lk_bcluster), LK_LINE);
-  size_t d_log = align_up(d_chist + (size_t)ctx->total * 256 * sizeof(uint32_t), LK_LINE);
+  size_t d_chist = align_up(d_bcl + (live ? ctx->C * sizeof(lk_bcluster) : 0), LK_LINE);
+  size_t d_bsm = align_up(d_chist + (live ? (size_t)ctx->total * 256 * sizeof(uint32_t) : 0), LK_LINE);
+  size_t d_log = align_up(d_bsm + ctx->G * sizeof(int32_t), LK_LINE);
   size_t dev_bytes = align_up(d_log + (size_t)ctx->G * ctx->log_cap * sizeof(lk_exec_rec), 4096);
   rc = lkb_alloc_device(ctx->device, dev_bytes, &ctx->dev_base);
   if (rc != LK_OK) return rc;
   char* db = (char*)ctx->dev_base;
-  /* control state starts at zero; the log records need no clearing */
-  rc = lkb_zero_device(ctx->device, db, d_log);
-  if (rc != LK_OK) return rc;
-  rc = lkb_copy_h2d(ctx->device, db + d_start, ctx->cl_start.data(), (ctx->C + 1) * sizeof(int32_t));
-  if (rc == LK_OK) rc = lkb_copy_h2d(ctx->device, db + d_rdoff, ctx->rd_off.data(), ctx->C * sizeof(int32_t));
-  if (rc == LK_OK && p->smids)
-    rc = lkb_copy_h2d(ctx->device, db + d_pin, p->smids, ctx->total * sizeof(int32_t));
-  if (rc != LK_OK) return rc;
+  char* head = mh + off_head;
+  ctx->head_h = head;
+  memcpy(head + d_start, ctx->cl_start.data(), (ctx->C + 1) * sizeof(int32_t));
+  memcpy(head + d_rdoff, ctx->rd_off.data(), ctx->C * sizeof(int32_t));
+  if (p->smids) memcpy(head + d_pin, p->smids, ctx->total * sizeof(int32_t));
 
   lk_kargs& a = ctx->args;
   memset(&a, 0, sizeof a);
@@ -394,9 +400,11 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   a.boot_count = (uint32_t*)(db + d_bcnt);
   a.log_count = (uint64_t*)(db + d_lcnt);
   a.log = ctx->log_cap ? (lk_exec_rec*)(db + d_log) : nullptr;
-  a.bcl = (lk_bcluster*)(db + d_bcl);
-  a.cta_hist = (uint32_t*)(db + d_chist);
+  a.bcl = live ? (lk_bcluster*)(db + d_bcl) : nullptr;
+  a.cta_hist = live ? (uint32_t*)(db + d_chist) : nullptr;
   a.crit_active = (int32_t*)(db + d_crit);
+  a.zero_base = db + d_dcl;
+  a.zero_bytes = d_bsm - d_dcl;
   a.num_clusters = ctx->C;
   a.grid = ctx->G;
   a.total = ctx->total;
@@ -417,7 +425,7 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   a.backoff_cap_ns = p->backoff_cap_ns ? p->backoff_cap_ns : 256;
   a.lease_ns = p->idle_lease_ns ? p->idle_lease_ns : 10000000000ull;
   a.boot_timeout_ns = p->boot_timeout_ns ? p->boot_timeout_ns : 10000000000ull;
-  if (live) ctx->ring_h = (lk_wire*)(mh + off_ring);
+  ctx->ring_h = (lk_wire*)(live ? mh + off_ring : head);
 
   ctx->tail = new (std::nothrow) Tail[ctx->C];
   ctx->rearmed = new (std::nothrow) Tail[ctx->C];
@@ -471,7 +479,7 @@ int lk_init(lk_ctx** out, const lk_init_params* p) {
   int rc = setup(ctx, p, true, 0);
   if (rc != LK_OK) { teardown(ctx); return rc; }
   beat(ctx);
-  rc = lkb_launch_kernel(ctx->device, &ctx->args, ctx->T, &ctx->launch);
+  rc = lkb_launch_kernel(ctx->device, &ctx->args, ctx->T, ctx->dev_base, ctx->head_h, ctx->head_bytes, &ctx->launch);
   if (rc != LK_OK) { ctx->launch = nullptr; teardown(ctx); return rc; }
   /* boot: every CTA read %smid, joined its cluster and counted itself */
   uint64_t t0 = now_ns();
@@ -840,9 +848,8 @@ int lk_run_finite(const lk_init_params* p, const lk_desc* descs, const int* clus
   ctx->finite = true;
   int rc = setup(ctx, p, false, R);
   if (rc != LK_OK) { teardown(ctx); return rc; }
-  /* fill the ring on the host, then copy it into device memory */
-  std::vector<lk_wire> ring((size_t)ctx->C * R);
-  memset(ring.data(), 0, ring.size() * sizeof(lk_wire));
+  /* fill the ring's pinned copy, which the launch sends to device memory */
+  lk_wire* ring = ctx->ring_h;
   std::vector<uint64_t> t(ctx->C, 0);
   for (size_t i = 0; i < count; ++i) {
     int c = cluster_of[i];
@@ -854,10 +861,8 @@ int lk_run_finite(const lk_init_params* p, const lk_desc* descs, const int* clus
     write_slot(&ring[(size_t)c * R + t[c]], t[c], ctx->R_log2, LK_CMD_EXIT, nullptr, nullptr, nullptr, nullptr);
     ++t[c];
   }
-  rc = lkb_copy_h2d(ctx->device, ctx->args.ring, ring.data(), ring.size() * sizeof(lk_wire));
-  if (rc != LK_OK) { teardown(ctx); return rc; }
   beat(ctx);
-  rc = lkb_launch_kernel(ctx->device, &ctx->args, ctx->T, &ctx->launch);
+  rc = lkb_launch_kernel(ctx->device, &ctx->args, ctx->T, ctx->dev_base, ctx->head_h, ctx->head_bytes, &ctx->launch);
   if (rc != LK_OK) { ctx->launch = nullptr; teardown(ctx); return rc; }
   /* bounded: the lease ends an idle kernel; the abort ends a stuck one */
   uint64_t limit = ctx->args.lease_ns + ctx->args.boot_timeout_ns;
@@ -1171,9 +1176,18 @@ static int serve_queue(lk_ctx* ctx, const lk_request* reqs, size_t count, const 
   }
   if (!ctx_alive(ctx)) return LK_ESTATE;
 
-  /* device state at the start of the arena: zeroed (copy engine), then the
-   * header the serving CTAs read; the host-mapped rings start empty */
-  int rc = lkb_zero_device(ctx->device, p->arena, sbytes);
+  /* device state at the start of the arena (21 MB for 4,096 slots): zeroed by the CTAs of cluster 0,
+   * then the header the serving CTAs read */
+  uint64_t zero_seq = 0;
+  const lk_desc zd{LK_OP_ZERO, 0, sbytes, 0};
+  int rc = LK_EAGAIN;
+  for (const uint64_t tz = now_ns();;) {
+    rc = post(ctx, 0, LK_CMD_WORK + LK_OP_ZERO, &zd, nullptr, nullptr, p->arena, &zero_seq);
+    if (rc != LK_EAGAIN || !ctx_alive(ctx) || now_ns() - tz > timeout) break;
+    std::this_thread::yield();
+  }
+  if (rc == LK_OK) rc = lk_wait(ctx, zero_seq, timeout);
+  if (rc != LK_OK) return rc == LK_EAGAIN ? LK_ETIMEDOUT : rc;
   lk_qstate hdr;
   memset(&hdr, 0, sizeof hdr);
   hdr.units = ctx->q_units_d;
@@ -1183,10 +1197,29 @@ static int serve_queue(lk_ctx* ctx, const lk_request* reqs, size_t count, const 
   hdr.qmask = ctx->qn - 1;
   hdr.qlog2 = ctx->qlog2;
   hdr.nslots = nslots;
-  if (rc == LK_OK) rc = lkb_copy_h2d(ctx->device, p->arena, &hdr, sizeof hdr);
+  rc = lkb_copy_h2d(ctx->device, p->arena, &hdr, sizeof hdr);
   if (rc != LK_OK) return rc;
-  memset(ctx->q_units_h, 0, (size_t)ctx->qn * sizeof(lk_qunit));
-  memset(ctx->q_cq_h, 0, (size_t)ctx->qn * sizeof(uint64_t));
+  /* The host-mapped rings start empty: an entry must not carry a current lap tag before it is written.
+   * They are cleared as far as they can be read, ahead of use, during the first lap: a CTA probes the
+   * unit index it claimed, and claims end at most one per CTA beyond the published ones; the completion
+   * ring is read at one entry per admitted request at most. */
+  const uint64_t q_ahead = (uint64_t)ctx->total + 1;
+  uint64_t q_clear = 0, cq_clear = 0;
+  auto clear_rings = [&](uint64_t units, uint64_t reqs_in) {
+    const uint64_t u1 = std::min<uint64_t>(units + q_ahead + 256, ctx->qn);   /* 256 units early */
+    const uint64_t r1 = std::min<uint64_t>(reqs_in + 1, ctx->qn);
+    if (u1 > q_clear) {
+      const uint64_t to = std::min<uint64_t>(u1 + 256, ctx->qn);
+      memset((void*)&ctx->q_units_h[q_clear], 0, (size_t)(to - q_clear) * sizeof(lk_qunit));
+      q_clear = to;
+    }
+    if (r1 > cq_clear) {
+      const uint64_t to = std::min<uint64_t>(r1 + 1024, ctx->qn);
+      memset((void*)&ctx->q_cq_h[cq_clear], 0, (size_t)(to - cq_clear) * sizeof(uint64_t));
+      cq_clear = to;
+    }
+  };
+  clear_rings(0, 0);
   st_rel(ctx->q_close_h, (uint64_t)0);
   beat(ctx);
   /* one LK_OP_SERVE per cluster: every CTA becomes a worker of the queue */
@@ -1241,7 +1274,7 @@ static int serve_queue(lk_ctx* ctx, const lk_request* reqs, size_t count, const 
   std::vector<size_t> slot_req(nslots, 0);
   std::deque<size_t> waiting;    /* arrived, not admitted (FIFO) */
   std::deque<size_t> active;     /* admitted with units left to publish (round-robin) */
-  uint64_t held = 0, next_u = 0, acked = 0, cq_head = 0, last_beat = t0;
+  uint64_t held = 0, next_u = 0, acked = 0, cq_head = 0, admitted = 0, last_beat = t0;
   uint64_t unpublished = 0;         /* units of admitted requests not yet published */
   uint64_t unpublished_bytes = 0;   /* and their input bytes */
   uint64_t pub_bytes = 0;           /* input bytes of every published unit */
@@ -1286,6 +1319,7 @@ static int serve_queue(lk_ctx* ctx, const lk_request* reqs, size_t count, const 
       if (q.arena_out && !arena.alloc(q.out_bytes, &oo)) break;
       q.out_off = oo;
       q.out = q.arena_out ? out_base + oo : reqs[i].out;
+      clear_rings(next_u, ++admitted);
       q.slot = free_slots.back();
       free_slots.pop_back();
       slot_req[q.slot] = i;
@@ -1315,6 +1349,7 @@ static int serve_queue(lk_ctx* ctx, const lk_request* reqs, size_t count, const 
       active.pop_front();
       QReq& q = st[i];
       const lk_request& r = reqs[i];
+      clear_rings(next_u + 1, admitted);   /* before a CTA can claim the indices this unit lets it reach */
       lk_qunit* e = &ctx->q_units_h[next_u & (ctx->qn - 1)];
       const uint64_t tag = (((next_u >> ctx->qlog2) + 1) & 0xffffull) << LK_TAG_SHIFT;
       __atomic_thread_fence(__ATOMIC_RELEASE);   /* earlier host writes before the entry's words */

@@ -15,6 +15,7 @@ LK_PENDING, lk_wait's LK_ETIMEDOUT, lk_submit's LK_EAGAIN), which are returned.
 from __future__ import annotations
 
 import ctypes
+import operator
 import os
 import threading
 
@@ -68,6 +69,9 @@ class lk_desc(ctypes.Structure):
     _fields_ = [("op", ctypes.c_uint32), ("flags", ctypes.c_uint32), ("n", ctypes.c_uint64),
                 ("aux", ctypes.c_uint64)]
 
+
+DESC_DTYPE = np.dtype([("op", "<u4"), ("flags", "<u4"), ("n", "<u8"), ("aux", "<u8")])
+assert DESC_DTYPE.itemsize == ctypes.sizeof(lk_desc)
 
 EXEC_REC_DTYPE = np.dtype([("seq", "<u8"), ("cluster", "<u4"), ("rank", "<u4"), ("smid", "<u4"), ("op", "<u4"),
                            ("order", "<u8"), ("t_pick_ns", "<u8"), ("t_start_ns", "<u8"), ("t_end_ns", "<u8"),
@@ -397,26 +401,28 @@ def lk_run_finite(sizes, descs, cluster_of, in0=None, in1=None, out=None, log_ca
     """Finite mode: one launch runs the listed descriptors and returns.
     descs: list of (op, n).  Returns (elapsed_ms, exec log array)."""
     lib = load(fake)
-    p, keep = make_params(sizes, exec_log_cap=kw.pop("exec_log_cap", max(1, len(descs))), **kw)
+    # the launch's log can only be read through log_cap
+    p, keep = make_params(sizes, exec_log_cap=kw.pop("exec_log_cap", max(1, len(descs)) if log_cap else 0), **kw)
     cnt = len(descs)
-    D = (lk_desc * max(1, cnt))(*[lk_desc(op, 0, n, 0) for op, n in descs])
+    D = np.zeros(max(1, cnt), dtype=DESC_DTYPE)
+    D["op"][:cnt] = [operator.index(op) & 0xFFFFFFFF for op, _ in descs]
+    D["n"][:cnt] = [operator.index(n) & 0xFFFFFFFFFFFFFFFF for _, n in descs]
     C = (ctypes.c_int * max(1, cnt))(*cluster_of)
 
-    def ctas_of(i):
+    def need(i, k):
         c = int(cluster_of[i])
-        return sizes[c] if 0 <= c < len(sizes) else 0
+        return op_bytes(descs[i][0], descs[i][1], sizes[c] if 0 <= c < len(sizes) else 0)[k] if i < cnt else 0
 
     def arr(xs, k):
         if xs is None:
             return None
         return (ctypes.c_void_p * max(1, cnt))(
-            *[_checked(x, op_bytes(descs[i][0], descs[i][1], ctas_of(i))[k] if i < cnt else 0, f"descriptor {i}")
-              for i, x in enumerate(xs)])
+            *[x if type(x) is int else _checked(x, need(i, k), f"descriptor {i}") for i, x in enumerate(xs)])
 
     ms = ctypes.c_float(-1.0)
     logbuf = np.zeros(max(1, log_cap), dtype=EXEC_REC_DTYPE)
     ln = ctypes.c_size_t()
-    rc = lib.lk_run_finite(ctypes.byref(p), D, C, arr(in0, 0), arr(in1, 1), arr(out, 2), cnt, ctypes.byref(ms),
+    rc = lib.lk_run_finite(ctypes.byref(p), D.ctypes.data_as(ctypes.POINTER(lk_desc)), C, arr(in0, 0), arr(in1, 1), arr(out, 2), cnt, ctypes.byref(ms),
                            logbuf.ctypes.data if log_cap else None, log_cap, ctypes.byref(ln))
     if rc != LK_OK:
         raise LkError(rc, "lk_run_finite")
