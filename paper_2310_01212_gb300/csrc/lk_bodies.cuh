@@ -650,9 +650,10 @@ struct lk_cta {
   uint64_t t_end;                  /* when the last body ended                                     */
 };
 
-/* Where a histogram's counts go.  With `cta` null, every CTA adds its
- * counts into `acc` (zero at rest) and a combine copies it out afterwards
- * (split parts, ordinary launches).  With `cta` set (descriptor `seq` of a
+/* Where a histogram's counts go.  With both pointers null, this CTA counts all
+ * of it and stores the bins.  With `acc` set, every CTA adds its counts into
+ * it (zero at rest) and a combine copies it out afterwards (split parts,
+ * ordinary launches).  With `cta` set (descriptor `seq` of a
  * cluster), rank 0 clears the output itself and release-stores seq into the
  * slot's clear word, and every CTA adds its counts straight into the output
  * once it has acquired that word: no combine, and no CTA waits for another at
@@ -748,7 +749,8 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
   const uint4* in = reinterpret_cast<const uint4*>(d.in0);
   bool ok = true;
   const uint64_t total = end - beg;
-  uint32_t* acc = sink.cta ? reinterpret_cast<uint32_t*>(d.out) : sink.acc;
+  uint32_t* acc = sink.acc ? sink.acc : reinterpret_cast<uint32_t*>(d.out);
+  const bool alone = !sink.acc && !sink.cta;
   /* rank 0 of a cluster: the counts' targets start at zero;
    * the others add once they see it */
   auto clear_out = [&]() -> bool {
@@ -780,7 +782,8 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
     for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
       uint32_t s = 0;
       for (uint32_t w = 0; w < W; ++w) s += sh[w * 256 + v];
-      if (s) atomicAdd(&acc[v], s);
+      if (alone) acc[v] = s;
+      else if (s) atomicAdd(&acc[v], s);
     }
     return ok && ready;
   }
@@ -805,7 +808,8 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
     const bool ready = hist_out_ready(sink, pace.deadline);
     for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
       const uint32_t tot = hist_row_readout<copies>(tbl, v);
-      if (tot) atomicAdd(&acc[v], tot);
+      if (alone) acc[v] = tot;
+      else if (tot) atomicAdd(&acc[v], tot);
     }
     return ok && ready;
   } else {
@@ -849,16 +853,17 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
     const bool ready = hist_out_ready(sink, pace.deadline);
     for (uint32_t v = threadIdx.x; ready && v < 256; v += T) {
       const uint32_t tot = hist_readout<P>(sh, v);
-      if (tot) atomicAdd(&acc[v], tot);
+      if (alone) acc[v] = tot;
+      else if (tot) atomicAdd(&acc[v], tot);
     }
     return ok && ready;
   }
 }
 
-/* Rank 0: copy the accumulator out and return it to zero for reuse. */
-__device__ __forceinline__ void combine_hist(const lk_slot& d, uint32_t* acc) {
+/* Threads t of `stride`: copy the accumulator out and return it to zero for reuse. */
+__device__ __forceinline__ void combine_hist(const lk_slot& d, uint32_t* acc, uint32_t t, uint32_t stride) {
   int32_t* out = reinterpret_cast<int32_t*>(d.out);
-  for (uint32_t v = threadIdx.x; v < 256; v += blockDim.x) {
+  for (uint32_t v = t; v < 256; v += stride) {
     out[v] = (int32_t)__ldcg(acc + v);
     acc[v] = 0;
   }

@@ -448,12 +448,88 @@ __device__ __forceinline__ void log_record(const lk_kargs& a, const lk_cta* cta,
   a.log_count[blockIdx.x] = j + 1;
 }
 
+/* A claimed work unit, in shared memory: part `part` of `parts` of an item. */
+struct lk_work {
+  lk_slot it;
+  float* psum;        /* per-part sums of a split item           */
+  uint32_t* pbins;    /* accumulator of a split histogram        */
+  uint32_t* pdone;    /* parts finished                          */
+  uint32_t part, parts;
+  uint32_t rslot;     /* serve: the request's slot               */
+  int32_t take;       /* 0 claimed, 1 none left, else LK_DERR_*  */
+};
+
+/* One thread: claim the next unit of a batch (its table lies in pinned
+ * host-mapped memory: an atomic and a round trip over the host link). */
+__device__ __forceinline__ void claim_batch(lk_bcluster* bc, const lk_unit* units, uint64_t nunits, lk_work& w) {
+  const unsigned long long u = atomicAdd(&bc->ticket, 1ull);
+  w.take = u >= nunits;
+  if (u >= nunits) return;
+  const ulonglong2* p = reinterpret_cast<const ulonglong2*>(units + u);
+  const ulonglong2 v0 = __ldcv(p), v1 = __ldcv(p + 1), v2 = __ldcv(p + 2);
+  const uint32_t op = (uint32_t)(v1.y >> 56);
+  w.it.cmd = LK_CMD_WORK + op;
+  w.it.in0 = v0.x;
+  w.it.in1 = v0.y;
+  w.it.out = v1.x;
+  w.it.n = v1.y & LK_LOW48;
+  w.part = (uint32_t)(v2.x & 0xffu);
+  w.parts = (uint32_t)((v2.x >> 8) & 0xffu);
+  const uint64_t comb = v2.x >> 16;   /* combine slot + 1, 0 = none */
+  if (comb && op == LK_OP_SUM_F32) {
+    w.psum = bc->sums[comb - 1].partial;
+    w.pdone = &bc->sums[comb - 1].done;
+  } else if (comb && op == LK_OP_HIST_U8) {
+    w.pbins = bc->hists[comb - 1].bins;
+    w.pdone = &bc->hists[comb - 1].done;
+  }
+}
+
+/* One thread: ask L2 for the first bytes of a claimed unit's inputs, as far as
+ * the body's stages would hold them. */
+__device__ __forceinline__ void prefetch_unit(const lk_work& w) {
+  uint64_t units = w.it.n, bytes = 16, beg, end;
+  switch (w.it.cmd - LK_CMD_WORK) {
+    case LK_OP_ADD_I32: case LK_OP_COPY_I32: case LK_OP_SUM_F32: units >>= 2; break;
+    case LK_OP_HIST_U8: units >>= 4; break;
+    case LK_OP_GEMM64_F32: bytes = 16384; break;
+    default: return;
+  }
+  if (bytes == 16384 && units < w.parts) return;   /* tiles split by rows */
+  share(units, (int)w.part, (int)w.parts, beg, end);
+  const bool two = w.it.in1 != 0;
+  const uint64_t cap = two ? 65536u : 131072u, len = (end - beg) * bytes;
+  if (len == 0) return;
+  prefetch_l2(w.it.in0 + beg * bytes, (uint32_t)(len < cap ? len : cap));
+  if (two) prefetch_l2(w.it.in1 + beg * bytes, (uint32_t)(len < cap ? len : cap));
+}
+
+/* One warp, after the CTA finished its part: the last part of a split sum or
+ * histogram writes the result (sums in binary64 by combine_sum, as a cluster
+ * of `parts` CTAs would, so a split sum is bit-identical to it) and returns
+ * the combine state to zero. */
+__device__ __forceinline__ void finish_part(const lk_work& w, uint32_t lane) {
+  const uint32_t op = w.it.cmd - LK_CMD_WORK;
+  if (w.parts <= 1 || (op != LK_OP_SUM_F32 && op != LK_OP_HIST_U8)) return;
+  int last = 0;
+  if (lane == 0) {
+    __threadfence();
+    last = atomicAdd(w.pdone, 1u) == w.parts - 1;
+    if (last) __threadfence();
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  if (op == LK_OP_SUM_F32) combine_sum(w.it, w.psum, (int)w.parts, lane);
+  else combine_hist(w.it, w.pbins, lane, 32);
+  __syncwarp();
+  if (lane == 0) *w.pdone = 0;
+}
+
 /* Work units, claimed one at a time by each CTA of the cluster, for two
  * descriptors (one loop, so the bodies are inlined once for both):
- *   LK_OP_BATCH (lk_submit_batch): units from the batch's table in pinned
- *     host-mapped memory, claimed with the cluster's ticket; the batch ends
- *     when the table is exhausted.  Parts of a split sum or histogram
- *     combine through per-item state in the cluster's batch state.
+ *   LK_OP_BATCH (lk_submit_batch): units from the batch's table, claimed with
+ *     the cluster's ticket; the batch ends when the table is exhausted.  Parts
+ *     of a split sum or histogram combine through per-item state in the
+ *     cluster's batch state.
  *   LK_OP_SERVE (lk_serve's device queue): the CTAs of every serving
  *     cluster claim the next unit index from one device counter and wait
  *     for that entry of the host-mapped unit ring (serve_take), until the
@@ -462,157 +538,125 @@ __device__ __forceinline__ void log_record(const lk_kargs& a, const lk_cta* cta,
  *     system-scope fence.
  * A unit is one part of one item or request, run by this CTA with the
  * body's (part, parts) split, so a result depends only on the item and its
- * parts.  The last part to finish (an acquire-release counter) writes a
- * split result -- sums in binary64 by combine_sum, as a cluster of `parts`
- * CTAs would, so a split sum is bit-identical to it -- and returns the
- * state to zero.  Returns an LK_DERR_* code or 0. */
+ * parts; an item of a single part is written by its body.
+ * In a batch, beside a unit of at most LK_AHEAD_BYTES another thread claims
+ * the next one and asks L2 for its first bytes, and warp 1 finishes the part
+ * before: together 3 us that stood between two units.  Larger units are
+ * claimed when the CTA is free: a unit claimed ahead waits for this CTA
+ * however long it takes, and 512 KB are 12 us of one SM's share of HBM.
+ * 1,000 items of 4 KB to 4 MB in parts of at most 512 KB on 148 CTAs: 150 us,
+ * 138 us with both (largest units first included).  Single-part histograms and
+ * sums go straight to their output: no accumulator to add to and copy out.
+ * Paced and yielding batches claim when free too.  Returns an LK_DERR_* code
+ * or 0. */
+#define LK_AHEAD_BYTES (512u * 1024u)
 template <int MAXT, int P>
 __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, int c, int r, unsigned char* dsm,
                                          uint64_t* bars, uint32_t& phase, float* red) {
-  __shared__ uint64_t s_w[5];                    /* in0, in1, out, op << 56 | n, unused */
-  __shared__ int s_take;                         /* 0 unit claimed, 1 none left, else LK_DERR_* */
-  __shared__ uint32_t s_part, s_parts;
-  __shared__ float* s_psum;                      /* per-part sums of a split item */
-  __shared__ uint32_t* s_pbins;                  /* accumulator of a split histogram */
-  __shared__ uint32_t* s_pdone;                  /* parts finished (split items) */
-  __shared__ uint32_t s_rslot;                   /* serve: the request's slot */
-  __shared__ float s_part_sum;
+  __shared__ __align__(64) lk_work s_u[3];       /* unit i in [i mod 3]: finishing, running, claimed ahead */
   __shared__ int s_lastp;
   const bool serve = d.cmd == LK_CMD_WORK + LK_OP_SERVE;
-  uint32_t* my_hist = a.cta_hist + (size_t)(a.cl_start[c] + r) * 256u;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t claimer = blockDim.x >= 96 ? 64u : 32u;
   /* batch */
   lk_bcluster* bc = a.bcl + c;
   const lk_unit* units = reinterpret_cast<const lk_unit*>(d.in0);
   const uint64_t nunits = d.n;
   /* serve */
   lk_qstate* qs = reinterpret_cast<lk_qstate*>(d.in0);
-  lk_qunit* qunits = nullptr;
   uint64_t* cq = nullptr;
-  const uint64_t* qclose = nullptr;
-  lk_qslot* qslots = nullptr;
   uint64_t qmask = 0;
-  uint32_t qlog2 = 0, nslots = 0;
+  uint32_t qlog2 = 0;
   if (serve) {
-    qunits = reinterpret_cast<lk_qunit*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->units)));
     cq = reinterpret_cast<uint64_t*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->cq)));
-    qclose = reinterpret_cast<const uint64_t*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->close)));
-    qslots = reinterpret_cast<lk_qslot*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->slots)));
     qmask = __ldcg(reinterpret_cast<const unsigned long long*>(&qs->qmask));
     qlog2 = __ldcg(&qs->qlog2);
-    nslots = __ldcg(&qs->nslots);
   }
+  auto claim = [&](lk_work& w) {   /* one thread */
+    w.it.seq = d.seq;
+    w.it.flags = 0;
+    w.it.aux = 0;
+    if (!serve) {
+      claim_batch(bc, units, nunits, w);
+      return;
+    }
+    lk_qunit* qunits = reinterpret_cast<lk_qunit*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->units)));
+    const uint64_t* qclose = reinterpret_cast<const uint64_t*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->close)));
+    lk_qslot* qslots = reinterpret_cast<lk_qslot*>(__ldcg(reinterpret_cast<const unsigned long long*>(&qs->slots)));
+    const unsigned long long u = atomicAdd(&qs->head, 1ull);
+    uint64_t e[6];
+    w.take = serve_take(a, qlog2, qunits + (u & qmask), u, qclose, e);
+    w.it.cmd = LK_CMD_WORK + (uint32_t)((e[4] >> 32) & 0xffull);
+    w.it.in0 = e[0];
+    w.it.in1 = e[1];
+    w.it.out = e[2];
+    w.it.n = e[3];
+    w.part = (uint32_t)(e[4] & 0xffffu);
+    w.parts = (uint32_t)((e[4] >> 16) & 0xffffu);
+    w.rslot = (uint32_t)e[5];
+    if (!w.take && (w.rslot >= __ldcg(&qs->nslots) || w.parts < 1 || w.parts > LK_SERVE_MAX_PARTS || w.part >= w.parts))
+      w.take = LK_DERR_BADDESC;
+    if (!w.take) {
+      lk_qslot* sl = qslots + w.rslot;
+      w.psum = sl->partial;
+      w.pbins = sl->bins;
+      w.pdone = &sl->done;
+    }
+  };
   const uint64_t rate = serve ? 0 : cta_rate(d.aux, a.cl_start[c + 1] - a.cl_start[c]);
   const int32_t* gate = (d.flags & LK_DFLAG_YIELD) ? a.crit_active : nullptr;
-  for (;;) {
-    if (threadIdx.x == 0) {
-      uint64_t w[5] = {0, 0, 0, 0, 0};
-      int take = 0;
-      uint32_t part = 0, parts = 1;
-      if (serve) {
-        const unsigned long long u = atomicAdd(&qs->head, 1ull);
-        uint64_t e[6];
-        take = serve_take(a, qlog2, qunits + (u & qmask), u, qclose, e);
-        part = (uint32_t)(e[4] & 0xffffu);
-        parts = (uint32_t)((e[4] >> 16) & 0xffffu);
-        const uint32_t rslot = (uint32_t)e[5];
-        w[0] = e[0];
-        w[1] = e[1];
-        w[2] = e[2];
-        w[3] = ((e[4] >> 32) & 0xffull) << 56 | e[3];   /* op << 56 | n, as a batch unit */
-        if (!take && (rslot >= nslots || parts < 1 || parts > LK_SERVE_MAX_PARTS || part >= parts))
-          take = LK_DERR_BADDESC;
-        if (!take) {
-          lk_qslot* sl = qslots + rslot;
-          s_psum = sl->partial;
-          s_pbins = sl->bins;
-          s_pdone = &sl->done;
-          s_rslot = rslot;
-        }
-      } else {
-        const unsigned long long u = atomicAdd(&bc->ticket, 1ull);
-        if (u < nunits) {
-          const ulonglong2* p = reinterpret_cast<const ulonglong2*>(units + u);
-          const ulonglong2 v0 = __ldcv(p), v1 = __ldcv(p + 1), v2 = __ldcv(p + 2);
-          w[0] = v0.x; w[1] = v0.y; w[2] = v1.x; w[3] = v1.y;
-          part = (uint32_t)(v2.x & 0xffu);
-          parts = (uint32_t)((v2.x >> 8) & 0xffu);
-          const uint64_t comb = v2.x >> 16;   /* combine slot + 1, 0 = none */
-          const uint32_t op = (uint32_t)(w[3] >> 56);
-          if (comb && op == LK_OP_SUM_F32) {
-            s_psum = bc->sums[comb - 1].partial;
-            s_pdone = &bc->sums[comb - 1].done;
-          } else if (comb && op == LK_OP_HIST_U8) {
-            s_pbins = bc->hists[comb - 1].bins;
-            s_pdone = &bc->hists[comb - 1].done;
-          }
-        } else {
-          take = 1;
-        }
-      }
-      for (int i = 0; i < 5; ++i) s_w[i] = w[i];
-      s_part = part;
-      s_parts = parts;
-      s_take = take;
-    }
-    __syncthreads();
-    const int take = s_take;   /* CTA-uniform */
+  if (tid == 0) claim(s_u[0]);
+  __syncthreads();
+  for (uint32_t i = 0;; ++i) {
+    lk_work& u = s_u[i % 3u];
+    if (!serve && i > 0 && warp == 1) finish_part(s_u[(i + 2u) % 3u], lane);
+    const int take = u.take;   /* CTA-uniform */
     if (take) return take == 1 ? 0 : take;
-    const uint32_t op = (uint32_t)(s_w[3] >> 56);
-    const uint32_t part = s_part, parts = s_parts;
-    lk_slot it;
-    it.seq = d.seq;
-    it.cmd = LK_CMD_WORK + op;
-    it.flags = 0;
-    it.n = s_w[3] & LK_LOW48;
-    it.in0 = s_w[0];
-    it.in1 = s_w[1];
-    it.out = s_w[2];
-    it.aux = 0;
-    it.t_pick = 0;
-    const Pace deadline{gtime() + 2000000000ull, rate, gate};
-    bool ok = true;
-    if (op == LK_OP_SUM_F32) {
-      float* pout = parts > 1 ? s_psum + part : &s_part_sum;
-      ok = body_sum<P, (MAXT <= 256 && P == 1)>(it, (int)part, (int)parts, dsm, bars, phase, deadline, red, pout);
-    } else if (op == LK_OP_HIST_U8) {
-      ok = body_hist<P, (MAXT <= 256)>(it, (int)part, (int)parts, dsm, bars, phase, deadline,
-                        HistSink{parts > 1 ? s_pbins : my_hist, nullptr, 0});
-    } else {
-      ok = run_body<MAXT, P>(it, (int)part, (int)parts, dsm, bars, phase, red, nullptr, HistSink{}, rate, gate,
-                             (a.flags & LK_KFLAG_GEMM_FFMA) == 0) == 0;
+    const uint32_t op = u.it.cmd - LK_CMD_WORK;
+    const uint32_t part = u.part, parts = u.parts;
+    const uint64_t elem = op == LK_OP_ADD_I32 ? 8u : op == LK_OP_HIST_U8 ? 1u : op == LK_OP_GEMM64_F32 ? 32768u : 4u;
+    const bool ahead = !serve && !rate && !gate && u.it.n * elem <= (uint64_t)LK_AHEAD_BYTES * parts;
+    if (ahead && tid == claimer) {
+      lk_work& nx = s_u[(i + 1u) % 3u];
+      claim(nx);
+      if (!nx.take) prefetch_unit(nx);
     }
+    __syncwarp();
+    const bool ok =
+        run_body<MAXT, P>(u.it, (int)part, (int)parts, dsm, bars, phase, red,
+                          parts > 1 ? u.psum + part : reinterpret_cast<float*>(u.it.out),
+                          HistSink{parts > 1 ? u.pbins : nullptr, nullptr, 0}, rate, gate,
+                          (a.flags & LK_KFLAG_GEMM_FFMA) == 0) == 0;
     __syncthreads();
-    /* the last part of a split sum or histogram (a single part always is) finishes it */
-    const bool split = parts > 1 && (op == LK_OP_SUM_F32 || op == LK_OP_HIST_U8 || serve);
-    if (threadIdx.x == 0) {
-      s_lastp = 1;
-      if (split) {
-        __threadfence();
-        s_lastp = atomicAdd(s_pdone, 1u) == parts - 1;
-        if (s_lastp) __threadfence();
-      }
-    }
-    __syncthreads();
-    if (s_lastp) {
-      if (op == LK_OP_SUM_F32) {
-        if (parts > 1) combine_sum(it, s_psum, (int)parts, threadIdx.x);
-        else if (threadIdx.x == 0) *reinterpret_cast<float*>(it.out) = s_part_sum;
-      } else if (op == LK_OP_HIST_U8) {
-        combine_hist(it, parts > 1 ? s_pbins : my_hist);
+    if (!ok) return LK_DERR_STAGING;
+    if (serve) {
+      /* the request's last part (a single part always is) finishes it */
+      if (tid == 0) {
+        s_lastp = 1;
+        if (parts > 1) {
+          __threadfence();
+          s_lastp = atomicAdd(u.pdone, 1u) == parts - 1;
+          if (s_lastp) __threadfence();
+        }
       }
       __syncthreads();
-      if (threadIdx.x == 0) {
-        if (split) *s_pdone = 0;
-        if (serve) {
+      if (s_lastp) {
+        if (parts > 1 && op == LK_OP_SUM_F32) combine_sum(u.it, u.psum, (int)parts, tid);
+        else if (parts > 1 && op == LK_OP_HIST_U8) combine_hist(u.it, u.pbins, tid, blockDim.x);
+        __syncthreads();
+        if (tid == 0) {
+          if (parts > 1) *u.pdone = 0;
           /* every output write of the request before its completion entry */
           fence_acq_rel_sys();
           const unsigned long long pos = atomicAdd(&qs->cq_tail, 1ull);
-          st_relaxed_sys(cq + (pos & qmask), (((uint64_t)pos >> qlog2) + 1) << 32 | s_rslot);
+          st_relaxed_sys(cq + (pos & qmask), (((uint64_t)pos >> qlog2) + 1) << 32 | u.rslot);
         }
       }
     }
-    __syncthreads();   /* the shared claim words are rewritten by the next claim */
-    if (!ok) return LK_DERR_STAGING;
+    if (!ahead) {
+      if (tid == 0) claim(s_u[(i + 1u) % 3u]);
+      __syncthreads();
+    }
   }
 }
 
@@ -1049,7 +1093,7 @@ __global__ void __launch_bounds__(MAXT) lk_ordinary(const lk_slot d, lk_scratch*
   __syncthreads();
   if (s_last) {
     if (op == LK_OP_SUM_F32) combine_sum(d, sc->partial, S, threadIdx.x);
-    else combine_hist(d, sc->hist);
+    else combine_hist(d, sc->hist, threadIdx.x, blockDim.x);
     __syncthreads();
     if (threadIdx.x == 0) sc->counter = 0;
   }

@@ -266,7 +266,6 @@ typedef struct {
   lk_exec_rec* log;              /* [G][log_cap] device, or NULL                        */
   uint64_t* log_count;           /* [G] device: records written per CTA                 */
   lk_bcluster* bcl;              /* [C] device: batch tickets and combine state         */
-  uint32_t* cta_hist;            /* [total][256] device: single-part histogram bins     */
   int32_t* crit_active;          /* device: critical descriptors running (lk_set_role)  */
   void* zero_base;               /* device: state the kernel clears at boot (128-byte   */
   uint64_t zero_bytes;           /* aligned, a multiple of 16 bytes)                    */

@@ -12,7 +12,7 @@ end where it starts, and more than a relay ring of them in flight."""
 import numpy as np
 import pytest
 
-from gpu_util import gemm_ok, host, need_gpu, to_dev
+from gpu_util import gemm_ok, host, need_gpu, sum_ok, to_dev
 from paper_2310_01212_gb300 import lk, synth
 
 pytestmark = pytest.mark.gpu
@@ -89,3 +89,40 @@ def test_hist_clear_after_earlier_writers(torch_ready, oracle_lib, finite, per_s
     assert np.array_equal(host(buf)[256:512].astype(np.int64), oracle_lib.hist_u8(xs[-1]))
     for i in range(rounds):
         assert np.array_equal(host(apart)[i].astype(np.int64), oracle_lib.hist_u8(xs[i])), i
+
+
+def test_batch_units_around_the_claim_ahead_size(torch_ready, oracle_lib):
+    """Units just below and above the size up to which a CTA claims its next
+    unit beside the current one, split and whole, on few CTAs (many units
+    each), in the bounds-checking build."""
+    torch = torch_ready
+    k = 512 * 1024
+    rows, checks = [], []
+    sizes = [16, 4096 + 3, k - 16, k, k + 16, 2 * k + 7]
+    for rep in range(3):
+        for i, nb in enumerate(sizes):
+            x = synth.bytes_uniform(34, 10 * rep + i, nb)
+            f = synth.normal_f32(35, 10 * rep + i, nb // 4)
+            a = synth.int32_uniform(36, 10 * rep + i, nb // 8, -(1 << 20), 1 << 20)
+            parts = (1, 2, 5)[rep]
+            oh = torch.full((256,), -1, dtype=torch.int32, device="cuda")
+            os_ = torch.full((4,), float("nan"), device="cuda")
+            oa = torch.full((a.size,), -1, dtype=torch.int32, device="cuda")
+            da = to_dev(a)
+            rows += [(lk.LK_OP_HIST_U8, x.size, (to_dev(x),), oh, parts), (lk.LK_OP_SUM_F32, f.size, (to_dev(f),), os_, parts),
+                     (lk.LK_OP_ADD_I32, a.size, (da, da), oa, parts)]
+            checks += [(oh, x), (os_, f), (oa, a)]
+    items = lk.batch_items(rows)
+    torch.cuda.current_stream().synchronize()
+    with lk.lk_init([5], bounds=True, idle_lease_ns=5_000_000_000) as c:
+        for _ in range(3):                                   # the combine state returns to zero
+            h = lk.lk_submit_batch(c, 0, items)
+            assert lk.lk_wait(c, h) == lk.LK_OK, lk.lk_device_error(c)
+    for out, ref in checks:
+        if ref.dtype == np.uint8:
+            assert np.array_equal(host(out).astype(np.int64), oracle_lib.hist_u8(ref)), ref.size
+        elif ref.dtype == np.float32:
+            assert sum_ok(host(out)[0], ref, oracle_lib), ref.size
+        else:
+            assert np.array_equal(host(out), oracle_lib.add_i32(ref, ref)), ref.size
+    assert lk.lk_bounds_violations() == (0, 0)
