@@ -115,6 +115,20 @@ __device__ __forceinline__ void bar_arrive(uint32_t id, uint32_t threads) {
   asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
+/* bar_sync that also returns the AND of every participant's v. */
+__device__ __forceinline__ bool bar_sync_and(uint32_t id, uint32_t threads, bool v) {
+  uint32_t out;
+  asm volatile(
+      "{\n\t.reg .pred pi, po;\n\t"
+      "setp.ne.u32 pi, %1, 0;\n\t"
+      "barrier.cta.red.and.pred po, %2, %3, pi;\n\t"
+      "selp.u32 %0, 1, 0, po;\n\t}"
+      : "=r"(out)
+      : "r"((uint32_t)v), "r"(id), "r"(threads)
+      : "memory");
+  return out != 0;
+}
+
 /* Exponential back-off between polls.  base == 0 spins without sleeping. */
 struct Backoff {
   uint32_t ns, cap;
@@ -151,10 +165,6 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
           smem_addr(dst)),
       "l"(src), "r"(bytes), "r"(smem_addr(bar))
       : "memory");
-}
-/* ask L2 for `bytes` (a multiple of 16) at a 16-byte aligned address */
-__device__ __forceinline__ void prefetch_l2(uint64_t src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;

@@ -485,25 +485,6 @@ __device__ __forceinline__ void claim_batch(lk_bcluster* bc, const lk_unit* unit
   }
 }
 
-/* One thread: ask L2 for the first bytes of a claimed unit's inputs, as far as
- * the body's stages would hold them. */
-__device__ __forceinline__ void prefetch_unit(const lk_work& w) {
-  uint64_t units = w.it.n, bytes = 16, beg, end;
-  switch (w.it.cmd - LK_CMD_WORK) {
-    case LK_OP_ADD_I32: case LK_OP_COPY_I32: case LK_OP_SUM_F32: units >>= 2; break;
-    case LK_OP_HIST_U8: units >>= 4; break;
-    case LK_OP_GEMM64_F32: bytes = 16384; break;
-    default: return;
-  }
-  if (bytes == 16384 && units < w.parts) return;   /* tiles split by rows */
-  share(units, (int)w.part, (int)w.parts, beg, end);
-  const bool two = w.it.in1 != 0;
-  const uint64_t cap = two ? 65536u : 131072u, len = (end - beg) * bytes;
-  if (len == 0) return;
-  prefetch_l2(w.it.in0 + beg * bytes, (uint32_t)(len < cap ? len : cap));
-  if (two) prefetch_l2(w.it.in1 + beg * bytes, (uint32_t)(len < cap ? len : cap));
-}
-
 /* One warp, after the CTA finished its part: the last part of a split sum or
  * histogram writes the result (sums in binary64 by combine_sum, as a cluster
  * of `parts` CTAs would, so a split sum is bit-identical to it) and returns
@@ -540,12 +521,13 @@ __device__ __forceinline__ void finish_part(const lk_work& w, uint32_t lane) {
  * body's (part, parts) split, so a result depends only on the item and its
  * parts; an item of a single part is written by its body.
  * In a batch, beside a unit of at most LK_AHEAD_BYTES another thread claims
- * the next one and asks L2 for its first bytes, and warp 1 finishes the part
- * before: together 3 us that stood between two units.  Larger units are
+ * the next one, and warp 1 finishes the part before: together 2 us that stood
+ * between two units.  Larger units are
  * claimed when the CTA is free: a unit claimed ahead waits for this CTA
  * however long it takes, and 512 KB are 12 us of one SM's share of HBM.
  * 1,000 items of 4 KB to 4 MB in parts of at most 512 KB on 148 CTAs: 150 us,
- * 138 us with both (largest units first included).  Single-part histograms and
+ * 134 us with both (largest units first included); asking L2 for the next
+ * unit's first 128 KB as well made it 139, for all of it 146.  Single-part histograms and
  * sums go straight to their output: no accumulator to add to and copy out.
  * Paced and yielding batches claim when free too.  Returns an LK_DERR_* code
  * or 0. */
@@ -616,11 +598,7 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
     const uint32_t part = u.part, parts = u.parts;
     const uint64_t elem = op == LK_OP_ADD_I32 ? 8u : op == LK_OP_HIST_U8 ? 1u : op == LK_OP_GEMM64_F32 ? 32768u : 4u;
     const bool ahead = !serve && !rate && !gate && u.it.n * elem <= (uint64_t)LK_AHEAD_BYTES * parts;
-    if (ahead && tid == claimer) {
-      lk_work& nx = s_u[(i + 1u) % 3u];
-      claim(nx);
-      if (!nx.take) prefetch_unit(nx);
-    }
+    if (ahead && tid == claimer) claim(s_u[(i + 1u) % 3u]);
     __syncwarp();
     const bool ok =
         run_body<MAXT, P>(u.it, (int)part, (int)parts, dsm, bars, phase, red,
