@@ -28,8 +28,9 @@
  *             rank 0 adds the partials in rank order in binary64
  *   gemm64    64x64x64 float32 tiles staged into shared memory by TMA bulk
  *             copies.  Whole tiles (one CTA per SM, 256 threads): tcgen05
- *             tensor cores on split-bf16 operands.  Row blocks and other
- *             shapes: six 32 KB stages (three with two CTAs per SM), 4x4
+ *             tensor cores on split-bf16 operands, or (on request, or with
+ *             two CTAs per SM) packed FFMA in k order, four tiles at a time
+ *             (two).  Row blocks of split tiles and other block sizes: 4x4
  *             register micro-tiles, FFMA in k order
  * Used by the persistent kernel and by the ordinary-launch baseline kernels.
  */
@@ -1212,6 +1213,148 @@ __device__ __forceinline__ void ffma_block(const float* sA, const float* sB, flo
   }
 }
 
+/* Whole tiles on the FFMA path, 256 threads: G groups of NT threads each take
+ * every G-th tile of the share [beg, end), so while one group waits at the end
+ * of its tile or for the next the others compute.  A thread accumulates 8 rows
+ * x MC columns in packed float32 pairs (fma.rn.f32x2: two outputs a
+ * multiply-add, each rounded as by fmaf), so every output is still its 64
+ * products in k order.  Lane l of a warp takes column chunk l % 8 (and + 8 if
+ * MC = 8) and rows 8 (l / 8) ..: an 8-lane phase of a 128-bit read covers 128
+ * contiguous bytes of B, or one broadcast word of A.
+ * What bounds it is the FP32 pipe, 2,048 clocks a tile, about as long as the
+ * tile's 48 KB take of an SM's share of HBM (2,275): measured 2,940 clocks, 2 x
+ * 32,768 tiles on 152 CTAs in 637 us (5.05 TB/s).  With 4 x 4 outputs a thread,
+ * scalar fmaf and the whole CTA on one tile it was 4,480 and 950 us: twice the
+ * shared-memory reads and instructions an output, and a CTA barrier a tile.
+ * Two CTAs per SM (128 registers): 3.75 -> 3.96 TB/s.
+ * Stages are shared by the groups: tile u sits in stage (u - beg) % NST, and
+ * the group that used it refills it; s_issued counts the loads issued into a
+ * stage, since a parity wait is only sound one phase ahead. */
+__device__ __forceinline__ uint64_t pack2(float a) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& c, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+template <int P>
+__device__ __forceinline__ bool body_gemm_ffma_tiles(const lk_slot& d, uint64_t beg, uint64_t end, unsigned char* dsm,
+                                                     uint64_t* bars, uint32_t& phase, Pace pace) {
+  constexpr uint32_t G = P == 1 ? 4 : 2, NT = 256 / G, MC = P == 1 ? 8 : 4, NP = MC / 2;
+  constexpr int KU = P == 1 ? 4 : 1;   /* k chunks of 4 per loop trip (P = 1: 1, 2, 4, 16 gave 4.2, 4.8, 5.1, 4.5 TB/s) */
+  constexpr uint32_t NST = P == 1 ? LK_TC_SMEM / 32768u : SmemCfg<P>::gemm_stages;   /* 7 or 3 */
+  static_assert(NST <= LK_NUM_BARS && NST >= G, "one mbarrier per stage, a stage per group");
+  const float* A = reinterpret_cast<const float*>(d.in0) + beg * 4096;
+  const float* B = reinterpret_cast<const float*>(d.in1) + beg * 4096;
+  float* C = reinterpret_cast<float*>(d.out) + beg * 4096;
+  const uint32_t tiles = (uint32_t)(end - beg);
+  const uint32_t g = threadIdx.x / NT, lt = threadIdx.x % NT, gw = lt >> 5, lane = threadIdx.x & 31u;
+  /* P = 1: warp 0, 1 of a group take row groups 0-3, 4-7, all columns; P = 2: warps 2 i + j take row
+   * groups 4 i .. and column half j */
+  const uint32_t rg = (lane >> 3) + 4u * (MC == 8 ? gw : gw >> 1);
+  const uint32_t col = 4u * (lane & 7u) + (MC == 8 ? 0u : 32u * (gw & 1u));
+  constexpr uint64_t unit_bytes = 32768u;
+  const uint64_t deadline = pace.rate ? pace.deadline + tiles * unit_bytes * 1000u / pace.rate : pace.deadline;
+  const uint64_t t_first = pace.rate ? gtime() : 0;
+  __shared__ uint32_t s_issued[NST];
+  auto issue = [&](uint32_t u) {   /* one thread */
+    const uint32_t st = u % NST;
+    unsigned char* sa = dsm + st * 32768u;
+    fence_proxy_async_smem();
+    if (!LK_INB(u < tiles, LK_OOB_GEMM_LOAD) ||
+        !LK_INB((st + 1) * 32768u <= (P == 1 ? LK_TC_SMEM : SmemCfg<P>::dyn_bytes), LK_OOB_GEMM_SMEM)) {
+      mbar_expect_tx(&bars[st], 0u);   /* skipped: the phase completes with no bytes */
+      return;
+    }
+    mbar_expect_tx(&bars[st], 32768u);
+    bulk_g2s(sa, A + (uint64_t)u * 4096, 16384u, &bars[st]);
+    bulk_g2s(sa + 16384u, B + (uint64_t)u * 4096, 16384u, &bars[st]);
+  };
+  auto parity = [&](uint32_t st, uint32_t use) { return ((phase >> st) & 1u) ^ (use & 1u); };
+  __syncthreads();          /* every stage is free: the previous use ended with a barrier */
+  if (threadIdx.x == 0)
+    for (uint32_t st = 0; st < NST; ++st) {
+      if (st < tiles) issue(st);
+      s_issued[st] = st < tiles;
+    }
+  __syncthreads();
+  bool ok = true;
+  for (uint32_t u = g; u < tiles; u += G) {
+    const uint32_t st = u % NST, use = u / NST;
+    const volatile uint32_t* iss = s_issued;
+    for (uint32_t it = 0; ok && iss[st] < use + 1; ++it)
+      if ((it & 15) == 15 && gtime() > deadline) ok = false;
+    if (ok) ok = mbar_wait(&bars[st], parity(st, use), deadline);
+    const float* sA = reinterpret_cast<const float*>(dsm + st * 32768u) + rg * 512u;
+    const float* sB = reinterpret_cast<const float*>(dsm + st * 32768u + 16384u) + col;
+    uint64_t c[8][NP];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < (int)NP; ++j) c[i][j] = 0;
+    if (ok) {
+#pragma unroll(KU)
+      for (uint32_t k = 0; k < 64; k += 4) {
+        float4 a[8];
+        ulonglong2 b[4][NP / 2];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(sA + i * 64 + k);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int h = 0; h < (int)NP / 2; ++h)
+            b[q][h] = *reinterpret_cast<const ulonglong2*>(sB + (k + q) * 64 + 32 * h);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint64_t aa = pack2(q == 0 ? a[i].x : q == 1 ? a[i].y : q == 2 ? a[i].z : a[i].w);
+#pragma unroll
+            for (int h = 0; h < (int)NP / 2; ++h) {
+              fma2(c[i][2 * h], aa, b[q][h].x);
+              fma2(c[i][2 * h + 1], aa, b[q][h].y);
+            }
+          }
+      }
+    }
+    /* the group has read the stage (and agrees whether it arrived) */
+    if (!bar_sync_and(3u + g, NT, ok)) {
+      ok = false;
+      break;
+    }
+    if (lt == 0 && u + NST < tiles) {
+      if (pace.rate) sleep_until(t_first + (u + 1) * unit_bytes * 1000u / pace.rate);
+      issue(u + NST);
+      __threadfence_block();
+      atomicAdd(&s_issued[st], 1u);
+    }
+    float* ct = C + (uint64_t)u * 4096 + rg * 512u + col;
+    if (LK_INB(u < tiles && rg * 8u + 8u <= 64u && col + 4u + 32u * (NP / 2 - 1) <= 64u, LK_OOB_GEMM_STORE)) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int h = 0; h < (int)NP / 2; ++h)
+          *reinterpret_cast<ulonglong2*>(ct + i * 64 + 32 * h) = make_ulonglong2(c[i][2 * h], c[i][2 * h + 1]);
+    }
+  }
+  ok = __syncthreads_and(ok);
+  if (!ok) {
+    /* copies may still be in flight: let every issued one land (bounded) */
+    if (threadIdx.x == 0)
+      for (uint32_t st = 0; st < NST; ++st)
+        if (s_issued[st]) mbar_wait(&bars[st], parity(st, s_issued[st] - 1), deadline + 1000000000ull);
+    __syncthreads();
+    return false;
+  }
+#pragma unroll
+  for (uint32_t st = 0; st < NST; ++st) {
+    const uint32_t uses = tiles > st ? (tiles - st + NST - 1) / NST : 0;
+    phase ^= (uses & 1u) << st;
+  }
+  return true;
+}
+
 /* Returns false if a staging copy did not complete before the deadline.
  * `phase` holds one parity bit per stage and persists across descriptors;
  * `pace` paces the tile loads as in stream().  Whole tiles at 256 threads
@@ -1233,6 +1376,9 @@ __device__ __forceinline__ bool body_gemm(const lk_slot& d, int r, int S, float*
   share(tiles * U, r, S, beg, end);
   if (!LK_INB(end <= tiles * U, LK_OOB_SHARE)) end = beg;
   if (beg >= end) return true;
+  if constexpr (FULL_UNROLL || P == 2)   /* the kernels of at most 256 threads */
+    if (U == 1 && blockDim.x == 256)
+      return body_gemm_ffma_tiles<P>(d, beg, end, reinterpret_cast<unsigned char*>(sm), bars, phase, pace);
   const float* A = reinterpret_cast<const float*>(d.in0);
   const float* B = reinterpret_cast<const float*>(d.in1);
   float* C = reinterpret_cast<float*>(d.out);

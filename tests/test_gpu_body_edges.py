@@ -42,8 +42,14 @@ def test_hist_share_edges(torch_ready, oracle_lib, threads):
     assert lk.lk_bounds_violations() == (0, 0)
 
 
-@pytest.mark.parametrize("S", [1, 2])
-def test_gemm_tile_counts(torch_ready, oracle_lib, S):
+# the tensor cores (one CTA per SM), the packed FFMA path, and it with two CTAs per SM
+@pytest.mark.parametrize("S,per_sm,flags", [(1, 1, 0), (2, 1, 0), (1, 1, lk.LK_INIT_GEMM_FFMA), (2, 1, lk.LK_INIT_GEMM_FFMA),
+                                            (1, 2, 0), (2, 2, 0)])
+def test_gemm_tile_counts(torch_ready, oracle_lib, S, per_sm, flags):
+    """Every number of tiles around the wrap of the stages, buffers and groups.
+    The k-order check allows one element in a thousand: binary64 rounds the sum
+    once before float32 does, which differs from one rounding for 2^-29 of them
+    a step at most."""
     torch = torch_ready
     cases = []
     for i, t in enumerate(list(range(1, 11)) + [17]):
@@ -51,12 +57,18 @@ def test_gemm_tile_counts(torch_ready, oracle_lib, S):
         B = synth.normal_f32(32, 2 * i + 1, t * 4096).reshape(t, 64, 64)
         cases.append((A, B, to_dev(A), to_dev(B), torch.full((t, 64, 64), float("nan"), device="cuda")))
     torch.cuda.current_stream().synchronize()
-    with lk.lk_init([S], bounds=True, idle_lease_ns=5_000_000_000) as c:
+    with lk.lk_init([S], bounds=True, idle_lease_ns=5_000_000_000, ctas_per_sm=per_sm, flags=flags) as c:
         hs = [lk.lk_submit(c, 0, lk.LK_OP_GEMM64_F32, A.shape[0], (dA, dB), dC) for A, B, dA, dB, dC in cases]
         for h in hs:
             assert lk.lk_wait(c, h) == lk.LK_OK, lk.lk_device_error(c)
     for A, B, _, _, dC in cases:
         assert gemm_ok(host(dC), A, B, oracle_lib), A.shape
+        if (flags or per_sm == 2) and A.shape[0] >= S:   # fused multiply-adds in k order, bit for bit
+            want = np.zeros(A.shape, np.float64)
+            for k in range(64):   # a product of two floats is exact in binary64; its sum with a float rounds once there
+                want = (A[:, :, k:k + 1].astype(np.float64) * B[:, k:k + 1, :].astype(np.float64)
+                        + want).astype(np.float32).astype(np.float64)
+            assert np.mean(host(dC) != want.astype(np.float32)) < 1e-3, A.shape   # double rounding, rarely
     assert lk.lk_bounds_violations() == (0, 0)
 
 
