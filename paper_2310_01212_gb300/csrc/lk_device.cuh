@@ -106,6 +106,12 @@ __device__ __forceinline__ void red_relaxed_gpu_add_s32(int32_t* p, int32_t v) {
 }
 __device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
+/* Programmatic dependent launch: a kernel launched that way may start while
+ * the one before it in the stream still runs; it waits here until that one has
+ * finished and its writes are visible.  Both are no-ops otherwise. */
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 /* Named CTA barriers (id 1..15; 0 is __syncthreads): `threads` arrivals open
  * one; bar_sync waits for it, bar_arrive only counts in.  Whole warps only. */
 __device__ __forceinline__ void bar_sync(uint32_t id, uint32_t threads) {

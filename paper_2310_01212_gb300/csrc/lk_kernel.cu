@@ -974,14 +974,15 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       uint64_t t_done = 0;
       if (tid == 0) s_cta.t_end = gtime();
       const bool comb = op == LK_OP_SUM_F32 || op == LK_OP_BATCH;
-      if (comb) {
-        if (tid == 0 && !s_err)
-          s_last = S == 1 || atom_add_acq_rel_gpu(&dc->arrive[slot].count, 1u) == (uint32_t)(S - 1);
-        __syncthreads();
-        if (s_last) {   /* CTA-uniform after the barrier */
-          if (op == LK_OP_SUM_F32) combine_sum(d, dc->partial[slot], S, tid);
-          __syncthreads();   /* the combine's writes before thread 0's fence */
+      if (comb && warp == 0) {   /* warp 0 alone: it arrives, and combines a sum if it was the last */
+        int last = 0;
+        if (tid == 0 && !s_err) {
+          last = S == 1 || atom_add_acq_rel_gpu(&dc->arrive[slot].count, 1u) == (uint32_t)(S - 1);
+          s_last = last;
         }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last && op == LK_OP_SUM_F32) combine_sum(d, dc->partial[slot], S, tid);
+        __syncwarp();   /* the combine's write before thread 0's fence */
       }
       if (tid == 0 && !s_err) {
         /* every output write of this CTA (and of the combine, when this CTA
@@ -1053,21 +1054,25 @@ __global__ void __launch_bounds__(MAXT) lk_ordinary(const lk_slot d, lk_scratch*
   __shared__ int32_t s_last;
   const int r = blockIdx.x, S = gridDim.x;
   const uint32_t op = d.cmd - LK_CMD_WORK;
-  if (op == LK_OP_NOP) return;
+  grid_launch_next();   /* once every CTA is here the next launch may set itself up behind this one */
+  if (op == LK_OP_NOP) {
+    grid_wait();
+    return;
+  }
   /* the shared stage barriers and those of this block's warps, one per thread */
   if (threadIdx.x < LK_NUM_BARS + (blockDim.x >> 5) * LK_STAGES) {
     mbar_init(&s_bars[threadIdx.x], 1);
     fence_barrier_init();
   }
   __syncthreads();
+  grid_wait();   /* nothing above touches global memory */
   uint32_t phase = 0;
   run_body<MAXT, 1>(d, r, S, dsm, s_bars, phase, s_red, &sc->partial[r], HistSink{sc->hist, nullptr, 0}, 0, nullptr);
   if (op != LK_OP_SUM_F32 && op != LK_OP_HIST_U8) return;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_last = atom_add_acq_rel_gpu(&sc->counter, 1u) == (uint32_t)(S - 1);
-  }
+  /* the acquire-release arrival orders the CTA's partial or counts (behind the
+   * barrier) before it, and the last arriver's combine after every other's */
+  if (threadIdx.x == 0) s_last = atom_add_acq_rel_gpu(&sc->counter, 1u) == (uint32_t)(S - 1);
   __syncthreads();
   if (s_last) {
     if (op == LK_OP_SUM_F32) combine_sum(d, sc->partial, S, threadIdx.x);
@@ -1432,13 +1437,25 @@ void pin_cpu(int cpu) {
   CPU_SET(cpu % n, &set);
   pthread_setaffinity_np(pthread_self(), sizeof set, &set);
 }
-cudaError_t launch_ordinary(const lk_slot& d, int grid, int threads, lk_scratch* sc, cudaStream_t s) {
+/* `early`: as a programmatic dependent launch (see grid_wait): its set-up
+ * overlaps the end of the launch before it in the stream. */
+cudaError_t launch_ordinary(const lk_slot& d, int grid, int threads, lk_scratch* sc, cudaStream_t s, bool early = false) {
   const uint32_t op = d.cmd - LK_CMD_WORK;
-  const size_t smem = (op == LK_OP_NOP || op == LK_OP_SPIN) ? 0 : lk::body_smem_bytes(1);
-  if (threads <= 256) lk_ordinary<256><<<grid, threads, smem, s>>>(d, sc);
-  else if (threads <= 512) lk_ordinary<512><<<grid, threads, smem, s>>>(d, sc);
-  else lk_ordinary<1024><<<grid, threads, smem, s>>>(d, sc);
-  return cudaGetLastError();
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (op == LK_OP_NOP || op == LK_OP_SPIN) ? 0 : lk::body_smem_bytes(1);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = early ? 1 : 0;
+  const cudaError_t e = threads <= 256   ? cudaLaunchKernelEx(&cfg, lk_ordinary<256>, d, sc)
+                        : threads <= 512 ? cudaLaunchKernelEx(&cfg, lk_ordinary<512>, d, sc)
+                                         : cudaLaunchKernelEx(&cfg, lk_ordinary<1024>, d, sc);
+  const cudaError_t last = cudaGetLastError();
+  return e != cudaSuccess ? e : last;
 }
 }  // namespace
 
@@ -1688,7 +1705,7 @@ extern "C" int lk_launch_noalloc(int device, const lk_desc* d, const void* const
   sl.in0 = n_in > 0 ? (uint64_t)(uintptr_t)in[0] : 0;
   sl.in1 = n_in > 1 ? (uint64_t)(uintptr_t)in[1] : 0;
   sl.out = (uint64_t)(uintptr_t)out;
-  return launch_ordinary(sl, ctas, threads, (lk_scratch*)scratch, (cudaStream_t)stream) == cudaSuccess
+  return launch_ordinary(sl, ctas, threads, (lk_scratch*)scratch, (cudaStream_t)stream, true) == cudaSuccess
              ? LK_OK
              : LK_EDEVICE;
 }

@@ -138,3 +138,56 @@ def test_batch_units_around_the_claim_ahead_size(torch_ready, oracle_lib):
         else:
             assert np.array_equal(host(out), oracle_lib.add_i32(ref, ref)), ref.size
     assert lk.lk_bounds_violations() == (0, 0)
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_noalloc_launches_follow_one_another(torch_ready, oracle_lib, graph):
+    """Dependent launches back to back on one stream, each reading what the one
+    before wrote, with every body and a launch of another kernel between them;
+    as they are and replayed from a captured graph."""
+    torch = torch_ready
+    n = 300_007
+    a = synth.int32_uniform(37, 0, n, 0, 255)
+    da = to_dev(a)
+    y, z, w = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(3))
+    h = torch.zeros(256, dtype=torch.int32, device="cuda")
+    s = torch.zeros(4, device="cuda")
+    f = torch.zeros(n, device="cuda")
+
+    def go(op, m, ins, out, ctas):
+        rc = lk.lk_launch_noalloc(op, m, ins, out, ctas=ctas, stream=torch.cuda.current_stream().cuda_stream)
+        assert rc == lk.LK_OK, rc
+
+    def chain():
+        go(lk.LK_OP_COPY_I32, n, (da,), y, 152)
+        for _ in range(4):
+            go(lk.LK_OP_ADD_I32, n, (y, da), z, 37)
+            go(lk.LK_OP_NOP, 0, (), None, 4)
+            go(lk.LK_OP_COPY_I32, n, (z,), y, 300)
+        go(lk.LK_OP_HIST_U8, 4 * n, (y,), h, 152)
+        torch.add(y, 1, out=w)
+        f.copy_(w)
+        go(lk.LK_OP_SUM_F32, n, (f,), s, 152)
+        go(lk.LK_OP_COPY_I32, n, (w,), z, 19)
+
+    go(lk.LK_OP_NOP, 0, (), None, 1)          # the scratch is set up before any capture
+    if graph:
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            chain()
+        torch.cuda.current_stream().wait_stream(side)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            chain()
+        for _ in range(3):
+            z.zero_()
+            g.replay()
+    else:
+        for _ in range(20):
+            chain()
+    want = 5 * a
+    assert np.array_equal(host(y), want)
+    assert np.array_equal(host(z), want + 1)
+    assert np.array_equal(host(h).astype(np.int64), oracle_lib.hist_u8(want.astype("<i4").view(np.uint8)))
+    assert float(host(s)[0]) == pytest.approx(float((want + 1).sum()), rel=1e-4)
