@@ -425,8 +425,7 @@ __device__ __forceinline__ void hist_zero(uint32_t* sh, uint32_t words) {
  * row is 256 bytes, so byte 1 of a counter's address is the bin itself and
  * the other three bytes belong to the lane: one byte permute of the loaded
  * word and the lane's base makes each address (no add).  Lane l only touches
- * bank l.  The 16 bytes of one vector: every address is formed before the
- * first reduction, so the reductions issue back to back.
+ * bank l.  The addresses are formed four reductions ahead.
  * What bounds it is the shared-memory pipe: 512 bytes of input cost 16 warp
  * reductions, a 128-bit read per lane (4 wavefronts) and the TMA write of the
  * same bytes (4), 24 clocks or 21.3 bytes a clock.  Measured per SM: 20.4 with
@@ -435,15 +434,21 @@ __device__ __forceinline__ void hist_zero(uint32_t* sh, uint32_t words) {
  * Loads straight into registers instead of through the ring: 21.1 on 38 CTAs,
  * but 5.24 TB/s on 152, too few bytes in flight.  A second copy of the
  * counters only adds clearing and read-out. */
+__device__ __forceinline__ uint32_t row_addr(uint32_t w, uint32_t lane_addr, uint32_t sel) {
+  uint32_t r;
+  asm volatile("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(lane_addr), "r"(sel));
+  return r;
+}
 __device__ __forceinline__ void count16_row(uint32_t lane_addr, uint4 q) {
   const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-  uint32_t a[16];
+  uint32_t a[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int j = 0; j < 4; ++j) a[j] = row_addr(w[0], lane_addr, 0x7604u | ((uint32_t)j << 4));
 #pragma unroll
-    for (int b = 0; b < 4; ++b) a[4 * i + b] = __byte_perm(w[i], lane_addr, 0x7604u | ((uint32_t)b << 4));
-#pragma unroll
-  for (int j = 0; j < 16; ++j) asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(a[j]) : "memory");
+  for (int j = 0; j < 16; ++j) {
+    asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], 1;" ::"r"(a[j & 3]) : "memory");
+    if (j < 12) a[j & 3] = row_addr(w[(j >> 2) + 1], lane_addr, 0x7604u | ((uint32_t)(j & 3) << 4));
+  }
 }
 
 /* Shared-memory offset (from dsm) of the counter table, and of warp w's ring:
@@ -566,14 +571,13 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
     return __all_sync(0xffffffffu, mbar_wait(&wb[ch % LK_STAGES], parity(ch), deadline));
   };
   uint64_t ch = 0;
-  /* At most four warps (stages of 8 KB): whole chunks, in pairs of 2 KB
-   * batches (four vectors a lane), the next batch loaded before the current
+  /* At most eight warps (stages of 4 KB and more): whole chunks, in pairs of 2
+   * KB batches (four vectors a lane), the next batch loaded before the current
    * one's 64 reductions are issued (they are ordered asm, so loads placed
-   * after them would wait for them), across the stage wait too.  With few
-   * warps nothing else covers those latencies (128 threads: 4.65 -> 5.29
-   * TB/s over 3 x 1 GiB); eight warps cover them for each other and lose to
-   * the longer code (256 threads: 5.88 -> 5.72). */
-  const uint64_t nfull = stage_vec % 512u == 0 ? total / stage_vec : 0;
+   * after them would wait for them), across the stage wait too (against
+   * loading a batch, then counting it: 128 threads, 4.65 -> 5.35 TB/s over 3 x
+   * 1 GiB; 256 threads, 8 x 256 MiB in 422 -> 409 us). */
+  const uint64_t nfull = stage_vec % 256u == 0 ? total / stage_vec : 0;
   if (PAIRS && nfull && !failed) {   /* PAIRS: kernels of at most 256 threads, which have the registers */
     uint4 q0[4], q1[4];
     auto load4 = [&](uint4 (&q)[4], const uint4* s0) {
@@ -800,7 +804,7 @@ __device__ __forceinline__ bool body_hist(const lk_slot& d, int r, int S, unsign
       __syncthreads();
       return cleared;
     };
-    ok = pace.gate ? hist_warp_streams<P, PAIRS, true>(in, beg, end, dsm, bars, phase, lane_addr, pace, prepare)
+    ok = pace.gate ? hist_warp_streams<P, false, true>(in, beg, end, dsm, bars, phase, lane_addr, pace, prepare)
                    : hist_warp_streams<P, PAIRS, false>(in, beg, end, dsm, bars, phase, lane_addr, pace, prepare);
     if (tail)
       for (uint64_t j = nv * 16 + threadIdx.x; j < d.n; j += T)

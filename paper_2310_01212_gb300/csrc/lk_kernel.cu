@@ -1106,9 +1106,9 @@ namespace {
  * a launch.  nullptr if the device cannot be read. */
 const cudaDeviceProp* dev_props(int device) {
   static std::mutex mu;
-  static cudaDeviceProp props[64];
-  static bool known[64];
-  if (device < 0 || device >= 64) return nullptr;
+  static cudaDeviceProp props[256];
+  static bool known[256];
+  if (device < 0 || device >= 256) return nullptr;
   std::lock_guard<std::mutex> g(mu);
   if (!known[device]) {
     if (cudaGetDeviceProperties(&props[device], device) != cudaSuccess) return nullptr;
