@@ -721,10 +721,12 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
   const uint32_t tid = threadIdx.x;
 
   /* ---- boot: clear the control state, read %smid, exchange, join a
-   * cluster.  The state (45 KB a cluster, live contexts 350 KB and 1 KB a CTA
-   * more) is cleared by all CTAs before the grid barrier below; sent from
+   * cluster.  The state (45 KB a cluster, live contexts 350 KB more) is cleared by all CTAs before the grid barrier below; sent from
    * pageable host memory it took lk_run_finite 0.1 ms a cluster. */
   __shared__ int32_t s_sm, s_slot, s_pos;
+  const bool fin = (a.flags & LK_KFLAG_FINITE) != 0;   /* the host waits for the kernel alone: no boot or exit reports */
+  for (uint32_t i = tid; i < LK_ALL_BARS; i += blockDim.x) mbar_init(&s_bars[i], 1);
+  fence_barrier_init();
   {
     uint4* z = reinterpret_cast<uint4*>(a.zero_base);
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + tid; i < a.zero_bytes / 16u; i += (uint64_t)a.grid * blockDim.x)
@@ -759,26 +761,29 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
     for (int j = (int)tid; j < a.grid; j += (int)blockDim.x) all[j] = __ldcg(a.boot_smid + j);
     __syncthreads();
     const int32_t my_sm = s_sm;
-    int below = 0;
-    for (int j = (int)tid; j < (int)blockIdx.x; j += (int)blockDim.x) below += all[j] == my_sm;
-    if (below) atomicAdd(&s_slot, below);
-    __syncthreads();
-    const int my_slot = s_slot;
+    int my_slot = 0;
+    if (P > 1) {
+      int below = 0;
+      for (int j = (int)tid; j < (int)blockIdx.x; j += (int)blockDim.x) below += all[j] == my_sm;
+      if (below) atomicAdd(&s_slot, below);
+      __syncthreads();
+      my_slot = s_slot;
+    }
     if (!a.pin_smid) {
       int before = 0;
       for (int j = (int)tid; j < a.grid; j += (int)blockDim.x) {
         int sj = 0;
-        for (int q = 0; q < j; ++q) sj += all[q] == all[j];
+        for (int q = 0; P > 1 && q < j; ++q) sj += all[q] == all[j];
         before += (sj < my_slot) || (sj == my_slot && all[j] < my_sm);
       }
       if (before) atomicAdd(&s_pos, before);
     }
     __syncthreads();
   }
-  if (tid == 0) {
+  if (tid < 32) {
     const int err = s_err;
     const uint32_t sm = (uint32_t)s_sm;
-    int c = -1, rk = -1;
+    int c = -1, rk = -1, size = 0;
     if (!err) {
       int pos = -1;
       if (a.pin_smid) {
@@ -792,30 +797,43 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       } else {
         pos = s_pos < a.total ? s_pos : -1;
       }
-      if (pos >= 0) {
-        c = 0;
-        while (a.cl_start[c + 1] <= pos) ++c;
-        rk = pos - a.cl_start[c];
+      /* the cluster whose positions hold pos: 32 at a time, one lane each */
+      for (int base = 0; pos >= 0 && c < 0 && base < a.num_clusters; base += 32) {
+        const int k = base + (int)tid;
+        int lo = 0, hi = 0;
+        if (k < a.num_clusters) {
+          lo = a.cl_start[k];
+          hi = a.cl_start[k + 1];
+        }
+        const uint32_t mine = __ballot_sync(0xffffffffu, lo <= pos && pos < hi);
+        if (mine) {
+          const int w = __ffs((int)mine) - 1;
+          c = base + w;
+          rk = pos - __shfl_sync(0xffffffffu, lo, w);
+          size = __shfl_sync(0xffffffffu, hi - lo, w);
+        }
       }
     }
-    s_cta.cl = c;
-    s_cta.rank = rk;
-    s_cta.size = c >= 0 ? a.cl_start[c + 1] - a.cl_start[c] : 0;
-    s_cta.dc = a.dcl + (c >= 0 ? c : 0);
-    s_cta.done = a.rdone + (c >= 0 ? a.rd_off[c] + rk : 0);
-    lk_cta_info* inf = a.info + blockIdx.x;
-    st_relaxed_sys32(&inf->cluster, c);
-    st_relaxed_sys32(&inf->rank, rk);
-    st_relaxed_sys32(&inf->smid, (int32_t)sm);
-    st_relaxed_sys32(&inf->slot, s_slot);
-    if (err) {
-      set_error(a, c, (uint32_t)err);
-    } else if (rk == 0) {
-      st_relaxed_sys(&a.cword[c].status, LK_ST_INIT);
+    if (tid == 0) {
+      s_cta.cl = c;
+      s_cta.rank = rk;
+      s_cta.size = size;
+      s_cta.dc = a.dcl + (c >= 0 ? c : 0);
+      s_cta.done = a.rdone + (c >= 0 ? a.rd_off[c] + rk : 0);
+      if (!fin) {
+        lk_cta_info* inf = a.info + blockIdx.x;
+        st_relaxed_sys32(&inf->cluster, c);
+        st_relaxed_sys32(&inf->rank, rk);
+        st_relaxed_sys32(&inf->smid, (int32_t)sm);
+        st_relaxed_sys32(&inf->slot, s_slot);
+      }
+      if (err) {
+        set_error(a, c, (uint32_t)err);
+      } else if (rk == 0 && !fin) {
+        st_relaxed_sys(&a.cword[c].status, LK_ST_INIT);
+      }
+      if (!fin) red_release_sys_add(&a.ctrl->booted, 1u);
     }
-    for (uint32_t i = 0; i < LK_ALL_BARS; ++i) mbar_init(&s_bars[i], 1);
-    fence_barrier_init();
-    red_release_sys_add(&a.ctrl->booted, 1u);
   }
   __syncthreads();
   if (s_cta.cl < 0 || s_err) return;
@@ -1022,8 +1040,10 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       st_relaxed_sys(&a.cword[c].done, known_done);
       fence_acq_rel_sys();
     }
-    if (master) st_relaxed_sys(&a.cword[c].status, final_err ? LK_ST_ERROR : LK_ST_EXITED);
-    red_release_sys_add(&a.ctrl->exited, 1u);
+    if (!fin) {
+      if (master) st_relaxed_sys(&a.cword[c].status, final_err ? LK_ST_ERROR : LK_ST_EXITED);
+      red_release_sys_add(&a.ctrl->exited, 1u);
+    }
   }
 }
 
