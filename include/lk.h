@@ -272,7 +272,8 @@ int lk_wait(lk_ctx* ctx, lk_handle h, uint64_t timeout_ns);
  * item is split into `parts` work units (a unit = one part of one item, run
  * by one CTA); the cluster's CTAs claim units from an atomic ticket, so
  * items of uneven size spread over the cluster.  Parts of a sum or histogram
- * item are combined by the last part to finish (sums: binary64 in part
+ * item are combined by the last part to finish (largest units are claimed
+ * first; sums: binary64 in part
  * order, so a result depends only on the item's n, its parts and the block
  * size).  One completion covers the whole batch. */
 typedef struct {
@@ -425,7 +426,8 @@ uint64_t lk_serve_queue_state_bytes(uint32_t max_inflight);
  * (coalescing applies to CHUNKS only).  Outputs taken from the arena are
  * released when the request completes (read them before the next call
  * reuses the arena).  In QUEUE mode the context must have been created live
- * (lk_init) and nothing else may be posted to it during the call.
+ * (lk_init) and nothing else may be posted to it during the call; cluster 0
+ * first clears the queue's state (operation 11 in the execution log).
  * Returns LK_OK if every request finished, LK_EINVAL, LK_ENOMEM (a request
  * needs more arena or budget than exists), or the first error. */
 int lk_serve(lk_ctx* ctx, const lk_request* reqs, size_t count, const lk_serve_params* p,
@@ -576,7 +578,10 @@ int lk_dispose_timed(lk_ctx* ctx, uint64_t timeout_ns, float* kernel_ms);
  * It runs one descriptor as an ordinary kernel launch (the same bodies and
  * split as lk_baseline_run_trace: `ctas` CTAs of `threads` threads) on the
  * caller's `stream` (a cudaStream_t; NULL = the legacy default stream) and
- * returns without waiting.  Unlike every other entry point it calls no
+ * returns without waiting.  It is a programmatic dependent launch: its CTAs may
+ * start while the launch before it on the stream ends, and wait for that to
+ * finish before their first access to global memory, so the stream's order
+ * holds as ever (in a captured graph too).  Unlike every other entry point it calls no
  * cudaMalloc, cudaFree or other allocating routine: the scratch that the sum
  * and histogram bodies use to combine per-CTA results is one file-scope
  * device array of 5,248 bytes, so it suits callers that cannot allocate --

@@ -29,7 +29,6 @@ int  lkb_alloc_mapped(int device, size_t bytes, size_t zero_bytes, void** host, 
 void lkb_free_mapped(void* host);
 int  lkb_alloc_device(int device, size_t bytes, void** dev);           /* not zeroed */
 void lkb_free_device(void* dev);
-int  lkb_zero_device(int device, void* dev, size_t bytes);           /* copy engine, not SMs */
 int  lkb_copy_h2d(int device, void* dst, const void* src, size_t bytes);
 int  lkb_copy_d2h(int device, void* dst, const void* src, size_t bytes);
 /* Streams for the end-to-end trace mode (copies beside a running kernel). */

@@ -84,10 +84,6 @@ int lkb_alloc_device(int, size_t bytes, void** dev) {
   return LK_OK;
 }
 void lkb_free_device(void* dev) { free(dev); }
-int lkb_zero_device(int, void* dev, size_t bytes) {
-  memset(dev, 0, bytes);
-  return LK_OK;
-}
 int lkb_copy_h2d(int, void* dst, const void* src, size_t bytes) {
   memcpy(dst, src, bytes);
   return LK_OK;

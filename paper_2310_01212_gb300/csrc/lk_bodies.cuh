@@ -877,17 +877,20 @@ __device__ __forceinline__ void combine_hist(const lk_slot& d, uint32_t* acc, ui
 /* ---- the compute-bound loop (Sec. III) ----------------------------------- */
 __device__ __forceinline__ void body_spin(const lk_slot& d, int r, uint32_t* red) {
   uint32_t x = 65536u * (uint32_t)r + threadIdx.x + 1u;
-  /* eight dependent steps per trip: a one-step trip spends most of its time
-   * on the 64-bit counter and the back edge, not on the multiply-add chain */
+  /* 32 dependent steps per trip: the 64-bit counter and the back edge cost some
+   * ten clocks a trip (20k steps, eight per trip: 43 to 51 us, depending on the
+   * code around the loop; 32: 45).  Each step is an instruction of its own: left to
+   * the compiler, several are folded into one multiply-add. */
   const uint64_t n = d.n;
   uint64_t i = 0;
+  auto step = [&]() { asm volatile("mad.lo.u32 %0, %0, %1, %2;" : "+r"(x) : "r"(1664525u), "r"(1013904223u)); };
 #pragma unroll 1
-  for (; i + 8 <= n; i += 8) {
+  for (; i + 32 <= n; i += 32) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x = 1664525u * x + 1013904223u;
+    for (int j = 0; j < 32; ++j) step();
   }
 #pragma unroll 1
-  for (; i < n; ++i) x = 1664525u * x + 1013904223u;
+  for (; i < n; ++i) step();
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) x ^= __shfl_xor_sync(0xffffffffu, x, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;

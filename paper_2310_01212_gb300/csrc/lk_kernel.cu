@@ -15,10 +15,11 @@
  * through a device ring (with LK_INIT_DIRECT every CTA's thread 0 polls the
  * ring itself; with LK_INIT_MAILBOX the master runs the paper's one-deep
  * to_GPU / from_GPU handshake instead of the ring), and every CTA runs its
- * share.  Each CTA then release-stores its own finished count; rank 0 gathers
- * the counts, combines partial results and publishes the descriptor's
- * sequence number in the host-mapped `done` word (from_GPU =
- * THREAD_FINISHED; the status word itself in mailbox mode).
+ * share.  Each CTA publishes its own completion word in host-mapped memory;
+ * the last to arrive on a descriptor's slot combines a sum and frees the slot
+ * (in mailbox mode rank 0 gathers the others' flags and answers
+ * THREAD_FINISHED).  In finite mode (lk_run_finite) every CTA reads the ring,
+ * which lies in device memory, and finishes one descriptor beside the next.
  *
  * Every device-side wait is bounded: by an idle lease (refreshed by the
  * host's heartbeat), by the host's abort word, and by a stall deadline.  On
@@ -1239,22 +1240,6 @@ void give_back(void* key, bool mapped) {
   }
 }
 
-int zero_device(int device, void* dev, size_t bytes) {
-  /* a host->device copy of zeros runs on a copy engine, not on the SMs */
-  static std::vector<char> zeros;
-  static std::mutex mu;
-  std::lock_guard<std::mutex> g(mu);
-  const size_t chunk = 4u << 20;
-  if (zeros.size() < chunk) zeros.assign(chunk, 0);
-  cudaStream_t s = copy_stream(device);
-  for (size_t off = 0; off < bytes; off += chunk) {
-    size_t nb = std::min(chunk, bytes - off);
-    if (cudaMemcpyAsync((char*)dev + off, zeros.data(), nb, cudaMemcpyHostToDevice, s) != cudaSuccess)
-      return LK_EDEVICE;
-  }
-  return cudaStreamSynchronize(s) == cudaSuccess ? LK_OK : LK_EDEVICE;
-}
-
 }  // namespace
 
 struct lkb_launch {
@@ -1296,7 +1281,6 @@ int lkb_alloc_device(int device, size_t bytes, void** dev) {
 }
 void lkb_free_device(void* dev) { give_back(dev, false); }
 
-int lkb_zero_device(int device, void* dev, size_t bytes) { return zero_device(device, dev, bytes); }
 
 int lkb_copy_h2d(int device, void* dst, const void* src, size_t bytes) {
   cudaStream_t s = copy_stream(device);
