@@ -62,8 +62,6 @@ __device__ __forceinline__ int4 add4(int4 x, int4 y) {
 #define LK_SMEM_WORK (64u * 1024u)     /* histogram counters or GEMM stages   */
 #define LK_SMEM_STREAM (128u * 1024u)  /* streaming stages                    */
 #define LK_SMEM_DYN (LK_SMEM_WORK + LK_SMEM_STREAM)
-#define LK_TC_SMEM (224u * 1024u)      /* P = 1: the tensor-core GEMM and the histogram's table and rings */
-#define LK_STAGES 4u
 #define LK_GEMM_STAGE_FLOATS 8192u     /* one GEMM stage: A rows 16 KB + B tile 16 KB */
 #define LK_HIST_COPIES 1u              /* lane-private counter copies (32 KB each) */
 #define LK_NUM_BARS 8u                 /* mbarriers: one per stage; the tensor-core GEMM's MMA completion in 4, 5 */
@@ -451,13 +449,11 @@ __device__ __forceinline__ void count16_row(uint32_t lane_addr, uint4 q) {
   }
 }
 
-/* Shared-memory offset (from dsm) of the counter table, and of warp w's ring:
- * three quarters of the rings follow the table (96 KB), the others end where
- * it starts (32 KB). */
+/* Shared-memory offset (from dsm) of the counter table; the rings lie around
+ * it (lk_hist_ring_off). */
 __device__ __forceinline__ uint32_t hist_table_off(const unsigned char* dsm) {
   return ((smem_addr(dsm) + 0xffffu) & ~0xffffu) - smem_addr(dsm);
 }
-#define LK_HIST_TABLE 65536u
 
 /* Clear the counters of the copies in use (the first 128 * copies bytes of
  * each 256-byte row). */
@@ -503,12 +499,9 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
                                                   F&& before_count) {
   static_assert(P == 1, "the counter rows need one CTA per SM's shared memory");
   const uint32_t W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t quarter = (W + 3u) / 4u;                   /* rings before the table */
-  const uint32_t ring_bytes = 32768u / quarter;
-  const uint32_t stage_vec = ring_bytes / LK_STAGES / 16u;
+  const uint32_t stage_vec = lk_hist_stage_vecs(W);
   const uint32_t tbl = hist_table_off(dsm);
-  const uint32_t ring_off = warp < 3u * quarter ? tbl + LK_HIST_TABLE + warp * ring_bytes
-                                                : tbl - 32768u + (warp - 3u * quarter) * ring_bytes;
+  const uint32_t ring_off = lk_hist_ring_off(W, warp, tbl);
   uint4* ring = reinterpret_cast<uint4*>(dsm + ring_off);
   uint64_t* wb = bars + LK_NUM_BARS + warp * LK_STAGES;
   uint64_t wbeg, wend;
@@ -518,7 +511,8 @@ __device__ __forceinline__ bool hist_warp_streams(const uint4* in, uint64_t beg,
   /* the warp's part, its ring slice and barriers, and the farthest counter
    * address any byte can form (row 255 of this lane and copy) */
   if (!LK_INB(wbeg <= wend && wend <= end, LK_OOB_SHARE) ||
-      !LK_INB(tbl >= 32768u && ring_off + LK_STAGES * stage_vec * 16u <= LK_TC_SMEM &&
+      !LK_INB(tbl >= LK_HIST_QUARTER && ring_off + LK_STAGES * stage_vec * 16u <= LK_TC_SMEM &&
+                  (smem_addr(ring) & 15u) == 0 &&
                   (ring_off >= tbl + LK_HIST_TABLE || ring_off + LK_STAGES * stage_vec * 16u <= tbl) &&
                   LK_NUM_BARS + (warp + 1) * LK_STAGES <= LK_ALL_BARS, LK_OOB_STREAM_SMEM) ||
       !LK_INB(((lane_addr >> 8) & 0xffu) == 0 && lane_addr - smem_addr(dsm) >= tbl &&

@@ -156,6 +156,25 @@ typedef struct __attribute__((aligned(LK_LINE))) {
   float partial[LK_BCAST_DEPTH][LK_MAX_CTAS]; /* per-rank partial sums                  */
 } lk_dcluster;
 
+/* ---- the histogram's table and rings (one CTA per SM) ------------------- */
+/* Its counters: 64 KB that start on a 64 KB boundary of the shared window,
+ * `tbl` bytes into a CTA's LK_TC_SMEM.  Each of the CTA's `warps` warps has a
+ * ring of LK_STAGES stages: three quarters of the rings follow the table (96
+ * KB), the others end where it starts (32 KB).  A ring is the destination of
+ * bulk copies and of 128-bit reads, so it is a whole number of 16-byte
+ * vectors: the stage is rounded down, and the ring follows from it (9 to 12
+ * and 17 to 28 warps divide the 32 KB unevenly). */
+#define LK_TC_SMEM (224u * 1024u)      /* P = 1: the tensor-core GEMM and the histogram's table and rings */
+#define LK_STAGES 4u
+#define LK_HIST_TABLE 65536u
+#define LK_HIST_QUARTER 32768u
+LK_HD uint32_t lk_hist_quarter(uint32_t warps) { return (warps + 3u) / 4u; }   /* rings in a quarter */
+LK_HD uint32_t lk_hist_stage_vecs(uint32_t warps) { return LK_HIST_QUARTER / lk_hist_quarter(warps) / LK_STAGES / 16u; }
+LK_HD uint32_t lk_hist_ring_off(uint32_t warps, uint32_t warp, uint32_t tbl) {
+  const uint32_t ring_bytes = lk_hist_stage_vecs(warps) * LK_STAGES * 16u, before = 3u * lk_hist_quarter(warps);
+  return warp < before ? tbl + LK_HIST_TABLE + warp * ring_bytes : tbl - LK_HIST_QUARTER + (warp - before) * ring_bytes;
+}
+
 /* ---- batches (lk_submit_batch) ----------------------------------------- */
 /* One work unit = one part of one item; the host expands a batch's items
  * into a unit table in pinned host-mapped memory (48 bytes per unit). */
