@@ -500,6 +500,7 @@ __device__ __forceinline__ void finish_part(const lk_work& w, uint32_t lane) {
     if (last) __threadfence();
   }
   if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  __syncwarp();   /* lane 0's acquire orders every lane's reads below: a shuffle alone orders no memory */
   if (op == LK_OP_SUM_F32) combine_sum(w.it, w.psum, (int)w.parts, lane);
   else combine_hist(w.it, w.pbins, lane, 32);
   __syncwarp();
@@ -684,6 +685,7 @@ __device__ __noinline__ void finish_finite(const lk_kargs& a, const lk_cta* cta,
   uint64_t t_done = 0;
   if (last) {
     if (d.cmd == LK_CMD_WORK + LK_OP_SUM_F32) {
+      __syncwarp();   /* lane 0's acquire before every lane's reads */
       combine_sum(d, dc->partial[slot], S, lane);
       __syncwarp();
     }
@@ -1000,6 +1002,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
           s_last = last;
         }
         last = __shfl_sync(0xffffffffu, last, 0);
+        __syncwarp();   /* thread 0's acquire before every lane's reads */
         if (last && op == LK_OP_SUM_F32) combine_sum(d, dc->partial[slot], S, tid);
         __syncwarp();   /* the combine's write before thread 0's fence */
       }
