@@ -684,7 +684,7 @@ __device__ __noinline__ void finish_finite(const lk_kargs& a, const lk_cta* cta,
   last = __shfl_sync(0xffffffffu, last, 0);
   uint64_t t_done = 0;
   if (last) {
-    if (d.cmd == LK_CMD_WORK + LK_OP_SUM_F32) {
+    if (d.cmd == LK_CMD_WORK + LK_OP_SUM_F32 && S > 1) {
       __syncwarp();   /* lane 0's acquire before every lane's reads */
       combine_sum(d, dc->partial[slot], S, lane);
       __syncwarp();
@@ -941,9 +941,13 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
     /* ---- run this CTA's share ------------------------------------------ */
     typename SlotArg<(MAXT > 512)>::type d = dsc;
     const uint32_t op = d.cmd - LK_CMD_WORK;
+    /* A cluster of one CTA runs its descriptors strictly one after another, so
+     * in finite mode its sums are stored by the body: warp 1 would combine them
+     * beside the next body, which may read or write the same place. */
+    float* partial = overlap && S == 1 ? reinterpret_cast<float*>(d.out) : &dc->partial[slot][r];
     const int berr = (op == LK_OP_BATCH || op == LK_OP_SERVE)
                          ? do_units<MAXT, P>(a, d, c, r, dsm, s_bars, phase, s_red)
-                         : run_body<MAXT, P>(d, r, S, dsm, s_bars, phase, s_red, &dc->partial[slot][r],
+                         : run_body<MAXT, P>(d, r, S, dsm, s_bars, phase, s_red, partial,
                                              HistSink{nullptr, &s_cta, d.seq},
                                              cta_rate(d.aux, S), (d.flags & LK_DFLAG_YIELD) ? a.crit_active : nullptr,
                                              (a.flags & LK_KFLAG_GEMM_FFMA) == 0);

@@ -1,0 +1,47 @@
+"""A cluster of one CTA runs its work strictly in order: what a descriptor
+wrote, the next one may read or overwrite."""
+import numpy as np
+import pytest
+
+from gpu_util import host, need_gpu
+from paper_2310_01212_gb300 import lk
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_ready(native_built):
+    return need_gpu()
+
+
+@pytest.mark.parametrize("per_sm,threads", [(1, 64), (1, 256), (2, 256), (1, 512)])
+@pytest.mark.parametrize("finite", [False, True])
+def test_a_sum_precedes_the_next_descriptor(torch_ready, finite, per_sm, threads):
+    """Sums into one word, each copied out by the next descriptor; and sums
+    whose word the next descriptor overwrites."""
+    torch = torch_ready
+    rounds, n = 300, 20_004
+    x = (torch.arange(rounds, device="cuda", dtype=torch.float32)[:, None] + 1).repeat(1, n).contiguous()
+    word = torch.zeros(4, device="cuda")                                  # read by the copy after it
+    seen = torch.full((rounds, 4), float("nan"), device="cuda")
+    over = torch.full((rounds, 4), float("nan"), device="cuda")           # overwritten by the copy after it
+    mark = torch.tensor([7, 8, 9, 10], dtype=torch.int32, device="cuda")
+    rows = []
+    for i in range(rounds):
+        rows.append((lk.LK_OP_SUM_F32, n, x[i], word))
+        rows.append((lk.LK_OP_COPY_I32, 4, word, seen[i]))
+        rows.append((lk.LK_OP_SUM_F32, n, x[i], over[i]))
+        rows.append((lk.LK_OP_COPY_I32, 4, mark, over[i]))
+    ptr = [(op, m, a.data_ptr(), o.data_ptr()) for op, m, a, o in rows]
+    torch.cuda.current_stream().synchronize()
+    if finite:
+        lk.lk_run_finite([1], [(op, m) for op, m, *_ in ptr], [0] * len(ptr), in0=[a for *_, a, _ in ptr],
+                         out=[o for *_, o in ptr], ctas_per_sm=per_sm, threads_per_cta=threads)
+    else:
+        with lk.lk_init([1], idle_lease_ns=5_000_000_000, ctas_per_sm=per_sm, threads_per_cta=threads,
+                        ring_depth=2048) as c:
+            hs = [lk.lk_submit(c, 0, op, m, (a,), o) for op, m, a, o in ptr]
+            assert all(h is not None for h in hs)
+            assert lk.lk_wait(c, hs[-1]) == lk.LK_OK, lk.lk_device_error(c)
+    assert np.array_equal(host(seen)[:, 0], np.float32(n) * np.arange(1, rounds + 1, dtype=np.float32))
+    assert np.array_equal(host(over).view(np.int32), np.tile(np.array([7, 8, 9, 10], np.int32), (rounds, 1)))
