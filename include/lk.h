@@ -272,10 +272,11 @@ int lk_wait(lk_ctx* ctx, lk_handle h, uint64_t timeout_ns);
  * item is split into `parts` work units (a unit = one part of one item, run
  * by one CTA); the cluster's CTAs claim units from an atomic ticket, so
  * items of uneven size spread over the cluster.  Parts of a sum or histogram
- * item are combined by the last part to finish (largest units are claimed
- * first; sums: binary64 in part
+ * item are combined by the last part to finish (sums: binary64 in part
  * order, so a result depends only on the item's n, its parts and the block
- * size).  One completion covers the whole batch. */
+ * size).  The largest units are claimed first and run beside one another, so
+ * items must not depend on each other, except on a cluster of one CTA, which
+ * runs them in the caller's order.  One completion covers the whole batch. */
 typedef struct {
   const void* in0;        /* device pointers, as lk_submit                        */
   const void* in1;

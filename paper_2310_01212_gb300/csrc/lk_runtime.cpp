@@ -691,12 +691,15 @@ int lk_submit_batch(lk_ctx* ctx, int cluster, const lk_batch_item* items, uint32
   /* Units go out largest first (by quarter octaves of their input bytes, items
    * of one size in the caller's order): a large unit claimed last would run
    * alone.  Adds and sums of up to 128 MB in 8 parts, 400 to a batch: CTAs
-   * ended between 688 and 864 us, now between 762 and 772 */
+   * ended between 688 and 864 us, now between 762 and 772.  On a cluster of one
+   * CTA there is nothing to balance: it runs the items in the caller's order. */
   auto parts_of = [&](const lk_batch_item& it) -> uint32_t {
     return it.parts ? std::min(it.parts, cap)
                     : (uint32_t)std::min<uint64_t>(cap, std::max<uint64_t>(1, (item_input_bytes(it.op, it.n) + part_bytes - 1) / part_bytes));
   };
+  const bool by_size = ctx->sizes[cluster] > 1;
   auto size_class = [&](const lk_batch_item& it) -> uint32_t {   /* 0..255, larger for larger units */
+    if (!by_size) return 0;
     const uint64_t b = item_input_bytes(it.op, it.n) / parts_of(it);
     if (b < 4) return (uint32_t)b;
     const int e = 63 - __builtin_clzll(b);

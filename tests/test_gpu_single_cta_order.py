@@ -45,3 +45,28 @@ def test_a_sum_precedes_the_next_descriptor(torch_ready, finite, per_sm, threads
             assert lk.lk_wait(c, hs[-1]) == lk.LK_OK, lk.lk_device_error(c)
     assert np.array_equal(host(seen)[:, 0], np.float32(n) * np.arange(1, rounds + 1, dtype=np.float32))
     assert np.array_equal(host(over).view(np.int32), np.tile(np.array([7, 8, 9, 10], np.int32), (rounds, 1)))
+
+
+@pytest.mark.parametrize("per_sm,threads", [(1, 64), (1, 256), (2, 256), (1, 1024)])
+def test_a_batch_keeps_the_callers_order(torch_ready, per_sm, threads):
+    """A small item, then a larger one that reads what it wrote, and a small
+    one, then a larger one into the same place."""
+    torch = torch_ready
+    rounds, n = 40, 1000
+    x = torch.arange(rounds * n, device="cuda", dtype=torch.int32).view(rounds, n)
+    f = (torch.arange(rounds, device="cuda", dtype=torch.float32)[:, None] + 1).repeat(1, n).contiguous()
+    y = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    z = torch.full((rounds, n), -1, dtype=torch.int32, device="cuda")
+    w = torch.full((rounds, 4), float("nan"), device="cuda")
+    rows = []
+    for i in range(rounds):
+        rows.append((lk.LK_OP_COPY_I32, n, (x[i],), y))
+        rows.append((lk.LK_OP_ADD_I32, n, (x[i], y), z[i]))
+        rows.append((lk.LK_OP_COPY_I32, 4, (x[i],), w[i]))
+        rows.append((lk.LK_OP_SUM_F32, n, (f[i],), w[i]))
+    items = lk.batch_items(rows)
+    torch.cuda.current_stream().synchronize()
+    with lk.lk_init([1], idle_lease_ns=5_000_000_000, ctas_per_sm=per_sm, threads_per_cta=threads) as c:
+        assert lk.lk_wait(c, lk.lk_submit_batch(c, 0, items)) == lk.LK_OK, lk.lk_device_error(c)
+    assert np.array_equal(host(z), 2 * host(x))
+    assert np.array_equal(host(w)[:, 0], np.float32(n) * np.arange(1, rounds + 1, dtype=np.float32))
