@@ -37,9 +37,9 @@ int  lkb_memcpy_async(void* stream, void* dst, const void* src, size_t bytes, in
 int  lkb_stream_sync(void* stream);
 void lkb_stream_destroy(void* stream);
 /* Launch the persistent kernel: a->grid CTAs of `threads` threads.  Before it
- * runs, `head_bytes` at head_src (pinned host memory that stays as it is until
- * the kernel has booted) are copied to head_dst on its stream, without a wait;
- * at boot it clears a->zero_base[0 .. zero_bytes). */
+ * runs, `head_bytes` at head_src (host memory that stays as it is until the
+ * kernel has booted; pinned: no wait) are copied to head_dst on its stream; at
+ * boot it clears a->zero_base[0 .. zero_bytes). */
 int  lkb_launch_kernel(int device, const lk_kargs* a, int threads, void* head_dst, const void* head_src,
                        size_t head_bytes, lkb_launch** out);
 /* 1 = kernel returned, 0 = still running, < 0 = LK_EDEVICE. */

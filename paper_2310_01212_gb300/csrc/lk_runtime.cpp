@@ -76,7 +76,8 @@ struct lk_ctx {
   lk_cta_info* info_h = nullptr;
 
   void* dev_base = nullptr;
-  const char* head_h = nullptr;  /* pinned copy of the first head_bytes of dev_base, sent with the launch */
+  const char* head_h = nullptr;  /* host copy of the first head_bytes of dev_base, sent with the launch */
+  void* head_mem = nullptr;      /* it, if not part of mapped_h (long finite lists) */
   size_t head_bytes = 0;
   lk_kargs args{};
   uint32_t log_cap = 0;
@@ -329,8 +330,13 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   size_t d_pin = align_up(d_rdoff + ctx->C * sizeof(int32_t), LK_LINE);
   size_t d_bcnt = align_up(d_pin + (p->smids ? ctx->total : 0) * sizeof(int32_t), LK_LINE);
   ctx->head_bytes = align_up(d_bcnt + sizeof(uint32_t), LK_LINE);
+  /* Pinned memory goes back to the library's pool, not to the system: a long
+   * list's ring lies in ordinary memory instead, freed with the context (16 MB:
+   * 262,144 slots over all clusters; sending them is then a small part of
+   * running them, at 2.4 us a NOP) */
+  const bool pinned_head = ctx->head_bytes <= (16u << 20);
   size_t off_head = align_up(off_close + LK_LINE, LK_LINE);
-  size_t off_units = align_up(off_head + ctx->head_bytes, LK_LINE);
+  size_t off_units = align_up(off_head + (pinned_head ? ctx->head_bytes : 0), LK_LINE);
   size_t units_bytes = (size_t)ctx->C * LK_BATCH_BUFFERS * ctx->max_units * sizeof(lk_unit);
   /* the serving queue: unit ring, completion ring (live only) */
   ctx->qn = live ? (p->serve_units ? p->serve_units : 65536u) : 0u;
@@ -380,6 +386,11 @@ static int setup(lk_ctx* ctx, const lk_init_params* p, bool live, uint32_t ring_
   if (rc != LK_OK) return rc;
   char* db = (char*)ctx->dev_base;
   char* head = mh + off_head;
+  if (!pinned_head) {
+    ctx->head_mem = calloc(1, ctx->head_bytes);
+    if (!ctx->head_mem) return LK_ENOMEM;
+    head = (char*)ctx->head_mem;
+  }
   ctx->head_h = head;
   memcpy(head + d_start, ctx->cl_start.data(), (ctx->C + 1) * sizeof(int32_t));
   memcpy(head + d_rdoff, ctx->rd_off.data(), ctx->C * sizeof(int32_t));
@@ -440,6 +451,7 @@ static void teardown(lk_ctx* ctx) {
   if (ctx->launch) lkb_release(ctx->launch);
   if (ctx->dev_base) lkb_free_device(ctx->dev_base);
   if (ctx->mapped_h) lkb_free_mapped(ctx->mapped_h);
+  free(ctx->head_mem);
   delete[] ctx->tail;
   delete[] ctx->rearmed;
   delete[] ctx->rate;
@@ -871,7 +883,7 @@ int lk_run_finite(const lk_init_params* p, const lk_desc* descs, const int* clus
   ctx->finite = true;
   int rc = setup(ctx, p, false, R);
   if (rc != LK_OK) { teardown(ctx); return rc; }
-  /* fill the ring's pinned copy, which the launch sends to device memory */
+  /* fill the ring's host copy, which the launch sends to device memory */
   lk_wire* ring = ctx->ring_h;
   std::vector<uint64_t> t(ctx->C, 0);
   for (size_t i = 0; i < count; ++i) {
