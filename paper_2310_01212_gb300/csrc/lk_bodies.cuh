@@ -644,6 +644,8 @@ struct lk_cta {
   lk_slot taken[LK_BCAST_DEPTH];   /* descriptor k (0-based) in [k mod D]: the last D taken        */
   lk_dcluster* dc;                 /* its cluster's device state                                   */
   uint64_t* done;                  /* its host-visible completion word                             */
+  const uint64_t* abort;           /* the host's abort word                                        */
+  uint64_t patience;               /* wait_finished: limit without progress (ns), 0 = the body's   */
   int32_t cl, rank, size;          /* cluster (-1: none), rank in it, the cluster's CTAs           */
   uint64_t t_pick[2], t_start[2];  /* stamps of descriptor k in [k mod 2], for the execution log   */
   uint64_t t_end;                  /* when the last body ended                                     */
@@ -691,9 +693,29 @@ __device__ __forceinline__ bool touches(const lk_slot& e, uint64_t lo, uint64_t 
   return (e.in0 < hi && e.in0 + b0 > lo) || (e.in1 < hi && e.in1 + b1 > lo) || (e.out < hi && e.out + bo > lo);
 }
 
+/* One thread: wait until another CTA's word reaches `want`; false if it does
+ * not in time.  The limit is the body's deadline, except in finite lists whose
+ * CTAs read the ring themselves (`patience`): there this CTA may be up to eight
+ * descriptors ahead of the one it waits for, whose bodies do not count against
+ * this one, so the wait goes on while the cluster finishes descriptors. */
+__device__ __noinline__ bool wait_finished(const lk_cta* cta, const uint64_t* word, uint64_t want, uint64_t deadline) {
+  const uint64_t limit = cta->patience;
+  lk_patience p = {0, limit ? gtime() + limit : deadline};
+  for (uint32_t it = 1;; ++it) {
+    if (ld_acquire_gpu(word) >= want) return true;
+    if (it & 63u) continue;
+    uint64_t progress = 0;
+    if (limit) {
+      if (ld_relaxed_sys(cta->abort)) return false;
+      for (uint32_t i = 0; i < LK_BCAST_DEPTH; ++i) progress += ld_relaxed_gpu(&cta->dc->slot_done[i]);
+    }
+    if (lk_out_of_patience(&p, gtime(), progress, limit)) return false;
+  }
+}
+
 /* Rank 0, the whole CTA: wait for the earlier descriptors that touch the
  * output of descriptor `seq` (one lane of warp 0 each); false, on every
- * thread, if one did not finish by `deadline`. */
+ * thread, if one did not finish in time. */
 __device__ __noinline__ bool hist_may_clear(const lk_cta* cta, uint64_t seq, uint64_t deadline) {
   __shared__ int s_clear;
   if (threadIdx.x < 32) {
@@ -702,11 +724,7 @@ __device__ __noinline__ bool hist_may_clear(const lk_cta* cta, uint64_t seq, uin
     if (back < LK_BCAST_DEPTH && back <= k) {
       const uint32_t i = (uint32_t)((k - back) % LK_BCAST_DEPTH);
       if (touches(cta->taken[i], out, out + 1024))
-        for (uint32_t it = 0; ld_acquire_gpu(&cta->dc->slot_done[i]) < k - back + 1; ++it)
-          if ((it & 63u) == 63u && gtime() > deadline) {
-            ok = false;
-            break;
-          }
+        ok = wait_finished(cta, &cta->dc->slot_done[i], k - back + 1, deadline);
     }
     ok = __all_sync(0xffffffffu, ok);
     if (threadIdx.x == 0) s_clear = ok;
@@ -717,19 +735,12 @@ __device__ __noinline__ bool hist_may_clear(const lk_cta* cta, uint64_t seq, uin
 
 /* Thread 0 waits for rank 0's cleared output (with a sink that has one),
  * then the whole CTA synchronises; false, on every thread, if the word did
- * not arrive by `deadline`. */
+ * not arrive in time. */
 __device__ __forceinline__ bool hist_out_ready(const HistSink& sink, uint64_t deadline) {
   __shared__ int s_ready;
-  if (threadIdx.x == 0) {
-    int ready = 1;
-    if (sink.cta)
-      for (uint32_t it = 0; ld_acquire_gpu(sink.clear_word()) < sink.seq; ++it)
-        if ((it & 63u) == 63u && gtime() > deadline) {
-          ready = 0;
-          break;
-        }
-    s_ready = ready;
-  }
+  if (threadIdx.x == 0)
+    s_ready = !sink.cta || ld_acquire_gpu(sink.clear_word()) >= sink.seq ||
+              wait_finished(sink.cta, sink.clear_word(), sink.seq, deadline);
   __syncthreads();
   return s_ready != 0;
 }

@@ -822,6 +822,8 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       s_cta.rank = rk;
       s_cta.size = size;
       s_cta.dc = a.dcl + (c >= 0 ? c : 0);
+      s_cta.abort = &a.ctrl->abort;
+      s_cta.patience = fin && (a.flags & LK_KFLAG_DIRECT) ? a.lease_ns + 1000000000ull : 0;   /* as wait_word */
       s_cta.done = a.rdone + (c >= 0 ? a.rd_off[c] + rk : 0);
       if (!fin) {
         lk_cta_info* inf = a.info + blockIdx.x;

@@ -156,6 +156,22 @@ typedef struct __attribute__((aligned(LK_LINE))) {
   float partial[LK_BCAST_DEPTH][LK_MAX_CTAS]; /* per-rank partial sums                  */
 } lk_dcluster;
 
+/* ---- a wait on another CTA's progress ------------------------------------ */
+/* Time limit of a wait for a CTA that may be several descriptors behind: it
+ * runs out `limit` ns after the cluster's progress word last changed, however
+ * long the wait as a whole takes.  One call per periodic check, with `until`
+ * set to the wait's start + limit before the first; true = give up. */
+typedef struct {
+  uint64_t progress, until;
+} lk_patience;
+LK_HD int lk_out_of_patience(lk_patience* p, uint64_t now, uint64_t progress, uint64_t limit) {
+  if (progress != p->progress) {
+    p->progress = progress;
+    p->until = now + limit;
+  }
+  return now > p->until;
+}
+
 /* ---- the histogram's table and rings (one CTA per SM) ------------------- */
 /* Its counters: 64 KB that start on a 64 KB boundary of the shared window,
  * `tbl` bytes into a CTA's LK_TC_SMEM.  Each of the CTA's `warps` warps has a
