@@ -706,7 +706,7 @@ __device__ __noinline__ bool wait_finished(const lk_cta* cta, const uint64_t* wo
     if (it & 63u) continue;
     uint64_t progress = 0;
     if (limit) {
-      if (ld_relaxed_sys(cta->abort)) return false;
+      if (ld_relaxed_sys(cta->abort) || ld_relaxed_gpu(&cta->dc->gen) == LK_GEN_STOP) return false;
       for (uint32_t i = 0; i < LK_BCAST_DEPTH; ++i) progress += ld_relaxed_gpu(&cta->dc->slot_done[i]);
     }
     if (lk_out_of_patience(&p, gtime(), progress, limit)) return false;

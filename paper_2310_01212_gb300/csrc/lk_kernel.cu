@@ -46,8 +46,6 @@
 
 using namespace lk;
 
-#define LK_GEN_STOP 0xffffffffffffffffull
-
 /* ======================================================================= */
 /* device side                                                              */
 /* ======================================================================= */
@@ -254,24 +252,19 @@ __device__ __forceinline__ int take_from_relay(const lk_kargs& a, const lk_dclus
   return 0;
 }
 
-/* Wait until *word >= want (GPU scope): relay generation, device-side done.
- * `stop_on_max` treats LK_GEN_STOP as the master's stop signal (returns -1).
- * *seen (optional) receives the value that satisfied the wait. */
-__device__ __noinline__ int wait_word(const lk_kargs& a, const uint64_t* word, uint64_t want, bool stop_on_max,
-                                      uint64_t* seen = nullptr) {
+/* Wait until *word >= want (GPU scope): a descriptor's completion word in the
+ * cluster's state dc.  Returns 0, -1 (a CTA of the cluster stopped: LK_GEN_STOP,
+ * its reason is recorded) or an LK_DERR_* reason. */
+__device__ __noinline__ int wait_word(const lk_kargs& a, const lk_dcluster* dc, const uint64_t* word, uint64_t want) {
   Backoff bo(a.backoff_base_ns, a.backoff_cap_ns);
   uint64_t hb = ld_relaxed_sys(&a.ctrl->heartbeat);
   uint64_t t_last = gtime();
   const uint64_t limit = a.lease_ns + 1000000000ull;
   for (uint32_t it = 1;; ++it) {
-    const uint64_t g = ld_acquire_gpu(word);
-    if (stop_on_max && g == LK_GEN_STOP) return -1;
-    if (g >= want) {
-      if (seen) *seen = g;
-      return 0;
-    }
+    if (ld_acquire_gpu(word) >= want) return 0;
     if ((it & 255) == 0) {
       if (ld_relaxed_sys(&a.ctrl->abort)) return LK_DERR_ABORT;
+      if (ld_relaxed_gpu(&dc->gen) == LK_GEN_STOP) return -1;
       const uint64_t now = gtime();
       if (now - t_last > limit) {
         const uint64_t h = ld_relaxed_sys(&a.ctrl->heartbeat);
@@ -884,8 +877,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
        * (EXIT uses no slot there). */
       const bool self_gate = relay ? master : (!err && dsc.cmd != LK_CMD_EXIT);
       if (!err && self_gate && need && s_slot_seen < need) {
-        const int ww = wait_word(a, &dc->slot_done[slot], need, false);
-        err = ww < 0 ? LK_DERR_STALL : ww;
+        err = wait_word(a, dc, &dc->slot_done[slot], need);
       }
       /* a batch starts once every earlier descriptor of the cluster finished
        * (its ticket and combine state are then at rest): the latest user of
@@ -893,24 +885,21 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       if (!err && self_gate && dsc.cmd == LK_CMD_WORK + LK_OP_BATCH) {
         for (uint64_t j = 1; j <= k && j <= LK_BCAST_DEPTH && !err; ++j) {
           const uint64_t q = k - j;
-          const int ww = wait_word(a, &dc->slot_done[q % LK_BCAST_DEPTH], q + 1, false);
-          err = ww < 0 ? LK_DERR_STALL : ww;
+          err = wait_word(a, dc, &dc->slot_done[q % LK_BCAST_DEPTH], q + 1);
         }
       }
       /* a critical descriptor (lk_set_role) counts as running from here to
        * its last CTA's completion; yielding clusters read the count */
       if (!err && master && (dsc.flags & LK_DFLAG_CRITICAL) && dsc.cmd != LK_CMD_EXIT)
         red_relaxed_gpu_add_s32(a.crit_active, 1);
-      if (relay && master) {
-        if (!err) relay_publish(&dc->relay[slot], k, dsc);
-        else st_release_gpu(&dc->gen, LK_GEN_STOP);
-      }
+      if (relay && master && !err) relay_publish(&dc->relay[slot], k, dsc);
       if (err) {
         if (err > 0) {
-          set_error(a, c, (uint32_t)err);
+          set_error(a, c, (uint32_t)err);   /* the reason first: the others leave on the stop word */
+          if (master || !relay) st_release_gpu(&dc->gen, LK_GEN_STOP);
           final_err = err;
         } else {
-          final_err = LK_DERR_STALL;   /* master stopped; its reason is recorded */
+          final_err = LK_DERR_STALL;   /* another CTA stopped; its reason is recorded */
         }
         s_exit = 1;
       } else {
@@ -1037,7 +1026,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       if (tid == 0) {
         set_error(a, c, (uint32_t)s_err);
         final_err = s_err;
-        if (master && relay) st_release_gpu(&dc->gen, LK_GEN_STOP);
+        if (master || !relay) st_release_gpu(&dc->gen, LK_GEN_STOP);
       }
       break;
     }

@@ -143,8 +143,11 @@ typedef struct __attribute__((aligned(LK_LINE))) {
   uint8_t pad[LK_LINE - 4];
 } lk_line_counter;
 
+#define LK_GEN_STOP 0xffffffffffffffffull
+
 typedef struct __attribute__((aligned(LK_LINE))) {
-  uint64_t gen;                          /* LK_GEN_STOP once the master stopped         */
+  uint64_t gen;                          /* LK_GEN_STOP once the master stopped (or, where every CTA reads */
+                                         /* the ring, any CTA): waits on the cluster's state end           */
   uint8_t pad0[LK_LINE - 8];
   uint64_t slot_done[LK_BCAST_DEPTH];    /* seq of the last finished descriptor of slot */
   uint8_t pad1[LK_LINE - 8 * LK_BCAST_DEPTH];

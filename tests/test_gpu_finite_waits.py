@@ -1,5 +1,8 @@
 """Waits of finite lists, whose CTAs run up to eight descriptors ahead of the
-slowest one of their cluster."""
+slowest one of their cluster.  Only rank 0 sums histograms: read from host
+memory by many clusters at once, they make it slow."""
+import time
+
 import numpy as np
 import pytest
 
@@ -14,26 +17,62 @@ def torch_ready(native_built):
     return need_gpu()
 
 
-def test_a_histogram_waits_for_a_slow_rank_0(torch_ready, oracle_lib):
-    """Only rank 0 sums histograms; here seven times 512 MB, from host memory and
-    in 152 clusters at once, some 2.7 s.  The other CTA reaches the histogram
-    behind them at once and waits for rank 0 to clear its output."""
-    torch = torch_ready
-    C, n, apart = 152, 1 << 19, 4096                     # histograms each; clusters read 4 MB apart
-    hp = torch.zeros((n + C * apart, 256), dtype=torch.int32, pin_memory=True)
-    hp[::apart, 5] = 3
+APART = 4096          # histograms (4 MB) between where two clusters start to read
+
+
+@pytest.fixture(scope="module")
+def host_hists(torch_ready):
+    hp = torch_ready.zeros(((1 << 20) + 256 * APART, 256), dtype=torch_ready.int32, pin_memory=True)
+    hp[::APART, 5] = 3
+    return hp
+
+
+def test_a_histogram_waits_for_a_slow_rank_0(torch_ready, oracle_lib, host_hists):
+    """Seven sums of 512 MB in each of 152 clusters, some 2.7 s.  The other CTA
+    reaches the histogram behind them at once and waits for rank 0 to clear its
+    output."""
+    torch, hp = torch_ready, host_hists
+    C, n = 152, 1 << 19
     x = synth.bytes_uniform(51, 0, 1 << 16)
     dx = to_dev(x)
     out = torch.full((C, 8, 256), -1, dtype=torch.int32, device="cuda")
     rows = []
     for c in range(C):
-        rows += [(c, lk.LK_OP_COMBINE_HIST, n, hp.data_ptr() + c * apart * 1024, out[c, j].data_ptr()) for j in range(7)]
+        rows += [(c, lk.LK_OP_COMBINE_HIST, n, hp.data_ptr() + c * APART * 1024, out[c, j].data_ptr()) for j in range(7)]
         rows.append((c, lk.LK_OP_HIST_U8, x.size, dx.data_ptr(), out[c, 7].data_ptr()))
     torch.cuda.current_stream().synchronize()
     lk.lk_run_finite([2] * C, [(op, m) for _, op, m, _, _ in rows], [c for c, *_ in rows], in0=[a for *_, a, _ in rows],
                      out=[o for *_, o in rows], threads_per_cta=64, ctas_per_sm=2)
     got = host(out).astype(np.int64)
     sums = np.zeros(256, np.int64)
-    sums[5] = 3 * (n // apart)
+    sums[5] = 3 * (n // APART)
     assert np.array_equal(got[:, :7], np.broadcast_to(sums, (C, 7, 256)))
     assert np.array_equal(got[:, 7], np.broadcast_to(oracle_lib.hist_u8(x), (C, 256)))
+
+
+def test_a_cluster_stops_soon_after_one_of_its_ctas(torch_ready, host_hists):
+    """One sum of 1 GB in each of 256 clusters, more than a second; the other CTA
+    of the larger clusters waits for it eight descriptors on, and with no lease
+    gives up after that second.  Rank 0 must not wait out a second of its own
+    for it."""
+    torch, hp = torch_ready, host_hists
+    sizes, n = [2] * 48 + [1] * 208, 1 << 20
+    out = torch.zeros((256, 256), dtype=torch.int32, device="cuda")
+    torch.cuda.current_stream().synchronize()
+
+    def go(nops, **kw):
+        rows = [(c, lk.LK_OP_COMBINE_HIST, n, hp.data_ptr() + c * APART * 1024, out[c].data_ptr()) for c in range(256)]
+        rows += [(c, lk.LK_OP_NOP, 0, 0, 0) for c in range(48) for _ in range(nops)]
+        t = time.perf_counter()
+        lk.lk_run_finite(sizes, [(op, m) for _, op, m, _, _ in rows], [c for c, *_ in rows],
+                         in0=[a for *_, a, _ in rows], out=[o for *_, o in rows], threads_per_cta=64, ctas_per_sm=2, **kw)
+        return time.perf_counter() - t
+
+    alone = go(0)
+    if alone < 1.15:
+        pytest.skip("host memory is too fast here for rank 0 to be late")
+    t = time.perf_counter()
+    with pytest.raises(lk.LkError) as e:
+        go(40, idle_lease_ns=1)
+    assert e.value.code == lk.LK_EDEVICE
+    assert time.perf_counter() - t < alone + 0.5
