@@ -427,8 +427,9 @@ uint64_t lk_serve_queue_state_bytes(uint32_t max_inflight);
  * (coalescing applies to CHUNKS only).  Outputs taken from the arena are
  * released when the request completes (read them before the next call
  * reuses the arena).  In QUEUE mode the context must have been created live
- * (lk_init) and nothing else may be posted to it during the call; cluster 0
- * first clears the queue's state (operation 11 in the execution log).
+ * (lk_init) and nothing else may be posted to it during the call; a cluster
+ * with nothing to run first clears the queue's state (operation 11 in the
+ * execution log), or copies from the host do if all have work queued.
  * Returns LK_OK if every request finished, LK_EINVAL, LK_ENOMEM (a request
  * needs more arena or budget than exists), or the first error. */
 int lk_serve(lk_ctx* ctx, const lk_request* reqs, size_t count, const lk_serve_params* p,
