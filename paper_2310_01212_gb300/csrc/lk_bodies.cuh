@@ -1062,8 +1062,10 @@ __device__ __forceinline__ bool body_gemm_tc(const lk_slot& d, int r, int S, uns
   auto parity = [&](uint32_t bar, uint32_t k) { return ((phase >> bar) & 1u) ^ (k & 1u); };
   __shared__ uint32_t s_tmem;
   __syncthreads();          /* every stage is free: the previous use ended with a barrier */
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
+    fence_proxy_async_global();   /* earlier generic writes before these async reads */
     for (uint32_t u = 0; u < tiles && u < LK_TC_STAGES; ++u) issue(u);
+  }
   if (warp == 0) {
     __syncwarp();
     tmem_alloc(&s_tmem, LK_TC_COLS);
@@ -1285,11 +1287,13 @@ __device__ __forceinline__ bool body_gemm_ffma_tiles(const lk_slot& d, uint64_t 
   };
   auto parity = [&](uint32_t st, uint32_t use) { return ((phase >> st) & 1u) ^ (use & 1u); };
   __syncthreads();          /* every stage is free: the previous use ended with a barrier */
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
+    fence_proxy_async_global();   /* earlier generic writes before these async reads */
     for (uint32_t st = 0; st < NST; ++st) {
       if (st < tiles) issue(st);
       s_issued[st] = st < tiles;
     }
+  }
   __syncthreads();
   bool ok = true;
   for (uint32_t u = g; u < tiles; u += G) {
@@ -1415,8 +1419,10 @@ __device__ __forceinline__ bool body_gemm(const lk_slot& d, int r, int S, float*
   };
   __shared__ int s_staged;
   __syncthreads();          /* every stage is free: the previous use ended with a barrier */
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
+    fence_proxy_async_global();   /* earlier generic writes before these async reads */
     for (uint64_t u = beg; u < end && u < beg + nstages; ++u) issue(u);
+  }
   bool ok = true;
   for (uint64_t u = beg; u < end; ++u) {
     const uint32_t st = (uint32_t)((u - beg) % nstages);

@@ -3,8 +3,8 @@ wrote, the next one may read or overwrite."""
 import numpy as np
 import pytest
 
-from gpu_util import host, need_gpu
-from paper_2310_01212_gb300 import lk
+from gpu_util import gemm_ok, host, need_gpu, to_dev
+from paper_2310_01212_gb300 import lk, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +70,32 @@ def test_a_batch_keeps_the_callers_order(torch_ready, per_sm, threads):
         assert lk.lk_wait(c, lk.lk_submit_batch(c, 0, items)) == lk.LK_OK, lk.lk_device_error(c)
     assert np.array_equal(host(z), 2 * host(x))
     assert np.array_equal(host(w)[:, 0], np.float32(n) * np.arange(1, rounds + 1, dtype=np.float32))
+
+
+@pytest.mark.parametrize("per_sm,threads,flags", [(1, 256, 0), (1, 256, lk.LK_INIT_GEMM_FFMA), (2, 256, 0), (1, 512, 0)])
+@pytest.mark.parametrize("finite", [False, True])
+def test_gemm_reads_what_the_descriptor_before_wrote(torch_ready, oracle_lib, finite, per_sm, threads, flags):
+    """Tiles that an add stored with ordinary writes, read by bulk copies."""
+    torch = torch_ready
+    rounds, tiles = 40, 3
+    A = synth.normal_f32(61, 0, rounds * tiles * 4096).reshape(rounds, tiles, 64, 64)
+    B = synth.normal_f32(61, 1, tiles * 4096).reshape(tiles, 64, 64)
+    dA, dB = to_dev(A), to_dev(B)
+    zero = torch.zeros((tiles, 64, 64), dtype=torch.int32, device="cuda")
+    buf = torch.full((tiles, 64, 64), float("nan"), device="cuda")
+    C = torch.full((rounds, tiles, 64, 64), float("nan"), device="cuda")
+    rows = []
+    for i in range(rounds):
+        rows.append((lk.LK_OP_ADD_I32, tiles * 4096, dA[i].data_ptr(), zero.data_ptr(), buf.data_ptr()))   # the same bits
+        rows.append((lk.LK_OP_GEMM64_F32, tiles, buf.data_ptr(), dB.data_ptr(), C[i].data_ptr()))
+    torch.cuda.current_stream().synchronize()
+    if finite:
+        lk.lk_run_finite([1], [r[:2] for r in rows], [0] * len(rows), in0=[r[2] for r in rows], in1=[r[3] for r in rows],
+                         out=[r[4] for r in rows], ctas_per_sm=per_sm, threads_per_cta=threads, flags=flags)
+    else:
+        with lk.lk_init([1], idle_lease_ns=5_000_000_000, ctas_per_sm=per_sm, threads_per_cta=threads, flags=flags) as c:
+            hs = [lk.lk_submit(c, 0, op, m, (a, b), o) for op, m, a, b, o in rows]
+            assert lk.lk_wait(c, hs[-1]) == lk.LK_OK, lk.lk_device_error(c)
+    got = host(C)
+    for i in range(rounds):
+        assert gemm_ok(got[i], A[i], B, oracle_lib), i
