@@ -1065,8 +1065,13 @@ struct lk_scratch {
   float partial[LK_MAX_CTAS];
 };
 
+/* Small blocks have an instance of their own, told that one CTA to an SM is
+ * enough (its shared memory allows no second): it takes 118 registers where
+ * 73 are chosen otherwise.  16 MB of tiles on one CTA, 64 threads: 2,042 us ->
+ * 1,773; 128: 1,223 -> 1,149.  At 256 threads the same hint slowed histograms
+ * (387 -> 406 us on one CTA), and tiles run on the tensor cores there. */
 template <int MAXT>
-__global__ void __launch_bounds__(MAXT) lk_ordinary(const lk_slot d, lk_scratch* sc) {
+__global__ void __launch_bounds__(MAXT, MAXT <= 128) lk_ordinary(const lk_slot d, lk_scratch* sc) {
   extern __shared__ __align__(128) unsigned char dsm[];
   __shared__ float s_red[32];
   __shared__ __align__(8) uint64_t s_bars[LK_ALL_BARS];
@@ -1147,6 +1152,7 @@ void preload_all() {
     const void* fns[] = {(const void*)lk_persistent<256, 1>,  (const void*)lk_persistent<512, 1>,
                          (const void*)lk_persistent<1024, 1>, (const void*)lk_persistent<256, 2>,
                          (const void*)lk_finite,
+                         (const void*)lk_ordinary<128>,
                          (const void*)lk_ordinary<256>,
                          (const void*)lk_ordinary<512>,    (const void*)lk_ordinary<1024>,
                          (const void*)lk_pingpong_kernel};
@@ -1154,10 +1160,11 @@ void preload_all() {
       cudaError_t e = cudaFuncGetAttributes(&fa, f);
       if (e != cudaSuccess && g_preload_err == cudaSuccess) g_preload_err = e;
     }
-    /* ordinary launches of the histogram / GEMM bodies take 64 KB of shared memory */
-    const void* ord[] = {(const void*)lk_ordinary<256>, (const void*)lk_ordinary<512>, (const void*)lk_ordinary<1024>};
-    for (int i = 0; i < 3; ++i) {
-      cudaError_t e = cudaFuncSetAttribute(ord[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+    /* ordinary launches of a body take the bodies' 224 KB of shared memory */
+    const void* ord[] = {(const void*)lk_ordinary<128>, (const void*)lk_ordinary<256>, (const void*)lk_ordinary<512>,
+                         (const void*)lk_ordinary<1024>};
+    for (const void* f : ord) {
+      cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)lk::body_smem_bytes(1));
       if (e != cudaSuccess && g_preload_err == cudaSuccess) g_preload_err = e;
     }
@@ -1453,7 +1460,8 @@ cudaError_t launch_ordinary(const lk_slot& d, int grid, int threads, lk_scratch*
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = early ? 1 : 0;
-  const cudaError_t e = threads <= 256   ? cudaLaunchKernelEx(&cfg, lk_ordinary<256>, d, sc)
+  const cudaError_t e = threads <= 128   ? cudaLaunchKernelEx(&cfg, lk_ordinary<128>, d, sc)
+                        : threads <= 256 ? cudaLaunchKernelEx(&cfg, lk_ordinary<256>, d, sc)
                         : threads <= 512 ? cudaLaunchKernelEx(&cfg, lk_ordinary<512>, d, sc)
                                          : cudaLaunchKernelEx(&cfg, lk_ordinary<1024>, d, sc);
   const cudaError_t last = cudaGetLastError();
