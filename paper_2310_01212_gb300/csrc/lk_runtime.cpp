@@ -100,7 +100,9 @@ struct lk_ctx {
     std::mutex mu;
     uint64_t next = 0;                          /* batches posted so far */
     uint64_t seq_of[LK_BATCH_BUFFERS] = {0};    /* batch seq that last used each table */
-    std::unique_ptr<uint32_t[]> order;          /* [max_units] the items, largest units first (scratch) */
+    /* scratch, [max_units] each: the items, largest units first; an item's parts | size class << 8 */
+    std::unique_ptr<uint32_t[]> order;
+    std::unique_ptr<uint16_t[]> meta;
   };
   BatchState* batch = nullptr;   /* [C] */
 
@@ -673,58 +675,58 @@ int lk_submit_batch(lk_ctx* ctx, int cluster, const lk_batch_item* items, uint32
   const uint64_t part_bytes = tune && tune->part_bytes ? tune->part_bytes : (4ull << 20);
   if (cap > 8) return LK_EINVAL;
   cap = std::min<uint32_t>(cap, (uint32_t)ctx->sizes[cluster]);
-  /* validate and count units, split sums and split histograms */
+  if (count > ctx->max_units) return LK_EINVAL;   /* an item is a unit at least */
+  lk_ctx::BatchState& bs = ctx->batch[cluster];
+  std::lock_guard<std::mutex> g(bs.mu);
+  if (!bs.order) bs.order.reset(new (std::nothrow) uint32_t[ctx->max_units]);
+  if (!bs.meta) bs.meta.reset(new (std::nothrow) uint16_t[ctx->max_units]);
+  if (!bs.order || !bs.meta) return LK_ENOMEM;
+  /* Units go out largest first (by quarter octaves of their input bytes, items
+   * of one size in the caller's order): a large unit claimed last would run
+   * alone.  Adds and sums of up to 128 MB in 8 parts, 400 to a batch: CTAs
+   * ended between 688 and 864 us, now between 762 and 772.  On a cluster of one
+   * CTA there is nothing to balance: it runs the items in the caller's order. */
+  const bool by_size = ctx->sizes[cluster] > 1;
+  auto size_class = [](uint64_t b) -> uint32_t {   /* 0..255, larger for larger units */
+    if (b < 4) return (uint32_t)b;
+    const int e = 63 - __builtin_clzll(b);
+    return (uint32_t)(4 * (e - 1)) + (uint32_t)((b >> (e - 2)) & 3u);
+  };
+  /* validate, count units, split sums and split histograms, and the items of each size: once per item,
+   * with divisions for split items only (500 small items: 16 us in several passes, 5 now) */
   uint64_t units = 0;
   uint32_t sums = 0, hists = 0;
+  uint32_t first[257] = {0};
   for (uint32_t i = 0; i < count; ++i) {
     const lk_batch_item& it = items[i];
     lk_desc d{it.op, 0, it.n, 0};
     int rc = validate(&d, it.in0, it.in1, op_inputs(it.op), it.out);
     if (rc != LK_OK) return rc;
     if (it.parts > 8) return LK_EINVAL;
-    uint32_t parts = it.parts ? std::min(it.parts, cap)
-                              : (uint32_t)std::min<uint64_t>(cap, std::max<uint64_t>(1, (item_input_bytes(it.op, it.n) + part_bytes - 1) / part_bytes));
+    const uint64_t bytes = item_input_bytes(it.op, it.n);
+    uint32_t parts = it.parts ? std::min(it.parts, cap) : 1;
+    if (!it.parts && bytes > part_bytes) parts = (uint32_t)std::min<uint64_t>(cap, (bytes - 1) / part_bytes + 1);
     if (parts > 1 && it.op == LK_OP_SUM_F32) ++sums;
     if (parts > 1 && it.op == LK_OP_HIST_U8) ++hists;
     units += parts;
+    const uint32_t size = by_size ? size_class(parts > 1 ? bytes / parts : bytes) : 0;
+    bs.meta[i] = (uint16_t)(parts | size << 8);
+    first[256 - size]++;
   }
   if (units > ctx->max_units || sums > LK_BATCH_SPLIT_SUMS || hists > LK_BATCH_SPLIT_HISTS) return LK_EINVAL;
   if (!ctx_alive(ctx)) return LK_ESTATE;
   beat(ctx);
-  lk_ctx::BatchState& bs = ctx->batch[cluster];
-  std::lock_guard<std::mutex> g(bs.mu);
   const uint32_t b = (uint32_t)(bs.next % LK_BATCH_BUFFERS);
   if (cl_done(ctx, cluster) < bs.seq_of[b]) return LK_EAGAIN;   /* table still in use */
-  if (!bs.order) bs.order.reset(new (std::nothrow) uint32_t[ctx->max_units]);   /* count <= units <= max_units */
-  if (!bs.order) return LK_ENOMEM;
   lk_unit* tab = ctx->units_h + ((size_t)cluster * LK_BATCH_BUFFERS + b) * ctx->max_units;
   uint64_t u = 0;
   uint32_t s_slot = 0, h_slot = 0;
-  /* Units go out largest first (by quarter octaves of their input bytes, items
-   * of one size in the caller's order): a large unit claimed last would run
-   * alone.  Adds and sums of up to 128 MB in 8 parts, 400 to a batch: CTAs
-   * ended between 688 and 864 us, now between 762 and 772.  On a cluster of one
-   * CTA there is nothing to balance: it runs the items in the caller's order. */
-  auto parts_of = [&](const lk_batch_item& it) -> uint32_t {
-    return it.parts ? std::min(it.parts, cap)
-                    : (uint32_t)std::min<uint64_t>(cap, std::max<uint64_t>(1, (item_input_bytes(it.op, it.n) + part_bytes - 1) / part_bytes));
-  };
-  const bool by_size = ctx->sizes[cluster] > 1;
-  auto size_class = [&](const lk_batch_item& it) -> uint32_t {   /* 0..255, larger for larger units */
-    if (!by_size) return 0;
-    const uint64_t b = item_input_bytes(it.op, it.n) / parts_of(it);
-    if (b < 4) return (uint32_t)b;
-    const int e = 63 - __builtin_clzll(b);
-    return (uint32_t)(4 * (e - 1)) + (uint32_t)((b >> (e - 2)) & 3u);
-  };
-  uint32_t first[257] = {0};
-  for (uint32_t i = 0; i < count; ++i) first[256 - size_class(items[i])]++;
   for (int k = 1; k <= 256; ++k) first[k] += first[k - 1];
-  for (uint32_t i = 0; i < count; ++i) bs.order[first[255 - size_class(items[i])]++] = i;
+  for (uint32_t i = 0; i < count; ++i) bs.order[first[255 - (bs.meta[i] >> 8)]++] = i;
   for (uint32_t o = 0; o < count; ++o) {
     const uint32_t i = bs.order[o];
     const lk_batch_item& it = items[i];
-    const uint32_t parts = parts_of(it);
+    const uint32_t parts = bs.meta[i] & 0xffu;
     uint64_t comb = 0;
     if (parts > 1 && it.op == LK_OP_SUM_F32) comb = ++s_slot;
     if (parts > 1 && it.op == LK_OP_HIST_U8) comb = ++h_slot;
