@@ -515,17 +515,21 @@ __device__ __forceinline__ void finish_part(const lk_work& w, uint32_t lane) {
  * A unit is one part of one item or request, run by this CTA with the
  * body's (part, parts) split, so a result depends only on the item and its
  * parts; an item of a single part is written by its body.
- * In a batch, beside a unit of at most LK_AHEAD_BYTES another thread claims
- * the next one, and warp 1 finishes the part before: together 2 us that stood
- * between two units.  Larger units are
+ * In a batch warp 1 finishes a part beside the next unit, and, at up to 256
+ * threads, another thread claims the next unit beside one of at most
+ * LK_AHEAD_BYTES: together 2 us that stood between two units.  Larger units are
  * claimed when the CTA is free: a unit claimed ahead waits for this CTA
- * however long it takes, and 512 KB are 12 us of one SM's share of HBM.
+ * however long it takes, and 512 KB are 12 us of one SM's share of HBM (GEMM
+ * tiles off the tensor cores count by lk_gemm_work: by their bytes alone a
+ * mixed batch with two CTAs per SM took 107 us instead of 81).
  * 1,000 items of 4 KB to 4 MB in parts of at most 512 KB on 148 CTAs: 150 us,
  * 134 us with both (largest units first included); asking L2 for the next
- * unit's first 128 KB as well made it 139, for all of it 146.  Single-part histograms and
- * sums go straight to their output: no accumulator to add to and copy out.
- * Paced and yielding batches claim when free too.  Returns an LK_DERR_* code
- * or 0. */
+ * unit's first 128 KB as well made it 139, for all of it 146.  In the larger
+ * kernels the claim costs the bodies more registers than it gains: 384
+ * threads, tiles of 4 to 64 MB, 644 us with it and 585 without.  Single-part
+ * histograms and sums go straight to their output: no accumulator to add to
+ * and copy out.  Paced and yielding batches claim when free too.  Returns an
+ * LK_DERR_* code or 0. */
 #define LK_AHEAD_BYTES (512u * 1024u)
 template <int MAXT, int P>
 __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, int c, int r, unsigned char* dsm,
@@ -591,8 +595,12 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
     if (take) return take == 1 ? 0 : take;
     const uint32_t op = u.it.cmd - LK_CMD_WORK;
     const uint32_t part = u.part, parts = u.parts;
-    const uint64_t elem = op == LK_OP_ADD_I32 ? 8u : op == LK_OP_HIST_U8 ? 1u : op == LK_OP_GEMM64_F32 ? 32768u : 4u;
-    const bool ahead = !serve && !rate && !gate && u.it.n * elem <= (uint64_t)LK_AHEAD_BYTES * parts;
+    bool ahead = false;
+    if constexpr (MAXT <= 256) {
+      const uint64_t tile = 32768u * lk_gemm_work(blockDim.x, P, (a.flags & LK_KFLAG_GEMM_FFMA) != 0);
+      const uint64_t elem = op == LK_OP_ADD_I32 ? 8u : op == LK_OP_HIST_U8 ? 1u : op == LK_OP_GEMM64_F32 ? tile : 4u;
+      ahead = !serve && !rate && !gate && u.it.n * elem <= (uint64_t)LK_AHEAD_BYTES * parts;
+    }
     if (ahead && tid == claimer) claim(s_u[(i + 1u) % 3u]);
     __syncwarp();
     const bool ok =
@@ -630,26 +638,6 @@ __device__ __forceinline__ int run_units(const lk_kargs& a, const lk_slot& d, in
       if (tid == 0) claim(s_u[(i + 1u) % 3u]);
       __syncthreads();
     }
-  }
-}
-
-/* run_units, out of line in the 1,024-thread kernels: inlined, it shares the
- * dispatch loop's 64 registers. */
-template <int MAXT, int P>
-__device__ __noinline__ uint32_t call_units(const lk_kargs& a, const lk_slot& d, int c, int r, unsigned char* dsm,
-                                            uint64_t* bars, uint32_t phase, float* red) {
-  const int err = run_units<MAXT, P>(a, d, c, r, dsm, bars, phase, red);
-  return phase | (uint32_t)err << 16;
-}
-template <int MAXT, int P>
-__device__ __forceinline__ int do_units(const lk_kargs& a, const lk_slot& d, int c, int r, unsigned char* dsm,
-                                        uint64_t* bars, uint32_t& phase, float* red) {
-  if constexpr (MAXT > 512) {
-    const uint32_t ret = call_units<MAXT, P>(a, d, c, r, dsm, bars, phase, red);
-    phase = ret & 0xffffu;
-    return (int)(ret >> 16);
-  } else {
-    return run_units<MAXT, P>(a, d, c, r, dsm, bars, phase, red);
   }
 }
 
@@ -937,7 +925,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
      * beside the next body, which may read or write the same place. */
     float* partial = overlap && S == 1 ? reinterpret_cast<float*>(d.out) : &dc->partial[slot][r];
     const int berr = (op == LK_OP_BATCH || op == LK_OP_SERVE)
-                         ? do_units<MAXT, P>(a, d, c, r, dsm, s_bars, phase, s_red)
+                         ? run_units<MAXT, P>(a, d, c, r, dsm, s_bars, phase, s_red)
                          : run_body<MAXT, P>(d, r, S, dsm, s_bars, phase, s_red, partial,
                                              HistSink{nullptr, &s_cta, d.seq},
                                              cta_rate(d.aux, S), (d.flags & LK_DFLAG_YIELD) ? a.crit_active : nullptr,

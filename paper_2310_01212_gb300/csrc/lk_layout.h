@@ -228,6 +228,13 @@ typedef struct __attribute__((aligned(LK_LINE))) {
   lk_hist_state hists[LK_BATCH_SPLIT_HISTS];
 } lk_bcluster;
 
+/* How long a tile of the GEMM takes for its input bytes, in those of a stream:
+ * 1 on the tensor cores (256 threads, one CTA per SM), else 4 (FFMA; one CTA
+ * takes 1.5 to 4 us for the 32 KB that a stream passes in 0.75). */
+LK_HD uint32_t lk_gemm_work(uint32_t threads, uint32_t ctas_per_sm, int ffma) {
+  return threads == 256 && ctas_per_sm == 1 && !ffma ? 1u : 4u;
+}
+
 /* ---- the serving queue (lk_serve, LK_SERVE_QUEUE) ------------------------
  * The host publishes work units (parts of admitted requests) into a ring in
  * pinned host-mapped memory; every CTA of the serving clusters claims the

@@ -681,12 +681,14 @@ int lk_submit_batch(lk_ctx* ctx, int cluster, const lk_batch_item* items, uint32
   if (!bs.order) bs.order.reset(new (std::nothrow) uint32_t[ctx->max_units]);
   if (!bs.meta) bs.meta.reset(new (std::nothrow) uint16_t[ctx->max_units]);
   if (!bs.order || !bs.meta) return LK_ENOMEM;
-  /* Units go out largest first (by quarter octaves of their input bytes, items
-   * of one size in the caller's order): a large unit claimed last would run
+  /* Units go out largest first (by quarter octaves of their work: the input
+   * bytes, weighed by lk_gemm_work; items of one size in the caller's order): a
+   * large unit claimed last would run
    * alone.  Adds and sums of up to 128 MB in 8 parts, 400 to a batch: CTAs
    * ended between 688 and 864 us, now between 762 and 772.  On a cluster of one
    * CTA there is nothing to balance: it runs the items in the caller's order. */
   const bool by_size = ctx->sizes[cluster] > 1;
+  const uint64_t gemm_work = lk_gemm_work(ctx->T, ctx->per_sm, (ctx->args.flags & LK_KFLAG_GEMM_FFMA) != 0);
   auto size_class = [](uint64_t b) -> uint32_t {   /* 0..255, larger for larger units */
     if (b < 4) return (uint32_t)b;
     const int e = 63 - __builtin_clzll(b);
@@ -709,7 +711,8 @@ int lk_submit_batch(lk_ctx* ctx, int cluster, const lk_batch_item* items, uint32
     if (parts > 1 && it.op == LK_OP_SUM_F32) ++sums;
     if (parts > 1 && it.op == LK_OP_HIST_U8) ++hists;
     units += parts;
-    const uint32_t size = by_size ? size_class(parts > 1 ? bytes / parts : bytes) : 0;
+    const uint64_t work = it.op == LK_OP_GEMM64_F32 ? bytes * gemm_work : bytes;
+    const uint32_t size = by_size ? size_class(parts > 1 ? work / parts : work) : 0;
     bs.meta[i] = (uint16_t)(parts | size << 8);
     first[256 - size]++;
   }
