@@ -1240,7 +1240,10 @@ __device__ __forceinline__ void ffma_block(const float* sA, const float* sB, flo
  * 32,768 tiles on 152 CTAs in 637 us (5.05 TB/s).  With 4 x 4 outputs a thread,
  * scalar fmaf and the whole CTA on one tile it was 4,480 and 950 us: twice the
  * shared-memory reads and instructions an output, and a CTA barrier a tile.
- * Two CTAs per SM (128 registers): 3.75 -> 3.96 TB/s.
+ * Two CTAs per SM (128 registers): 3.75 -> 3.96 TB/s.  A share of one tile is
+ * left to the whole CTA (below), where one group alone would work on it: 24
+ * descriptors of one tile a CTA in 132 us instead of 159; of two tiles the
+ * groups take 171 and the whole CTA 182.
  * Stages are shared by the groups: tile u sits in stage (u - beg) % NST, and
  * the group that used it refills it; s_issued counts the loads issued into a
  * stage, since a parity wait is only sound one phase ahead. */
@@ -1393,7 +1396,7 @@ __device__ __forceinline__ bool body_gemm(const lk_slot& d, int r, int S, float*
   if (!LK_INB(end <= tiles * U, LK_OOB_SHARE)) end = beg;
   if (beg >= end) return true;
   if constexpr (FULL_UNROLL || P == 2)   /* the kernels of at most 256 threads */
-    if (U == 1 && blockDim.x == 256)
+    if (U == 1 && blockDim.x == 256 && end - beg > 1)
       return body_gemm_ffma_tiles<P>(d, beg, end, reinterpret_cast<unsigned char*>(sm), bars, phase, pace);
   const float* A = reinterpret_cast<const float*>(d.in0);
   const float* B = reinterpret_cast<const float*>(d.in1);
