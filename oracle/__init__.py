@@ -60,6 +60,7 @@ def lib() -> ctypes.CDLL:
             l.lko_abs_sum_f32.argtypes = [P, S]
             l.lko_abs_sum_f32.restype = ctypes.c_double
             l.lko_gemm64_f32.argtypes = [P, P, P, S]
+            l.lko_gemm64_fmaf.argtypes = [P, P, P, S]
             l.lko_gemm64_abs_bound.argtypes = [P, P, P, S]
             l.lko_spin_xor.argtypes = [ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint64]
             l.lko_spin_xor.restype = ctypes.c_uint32
@@ -117,6 +118,16 @@ def gemm64_f32(A: np.ndarray, B: np.ndarray) -> np.ndarray:
     assert A.shape == B.shape and A.shape[-2:] == (64, 64)
     C = np.empty(A.shape, dtype=np.float64)
     lib().lko_gemm64_f32(_p(A), _p(B), _p(C), A.size // 4096)
+    return C
+
+
+def gemm64_fmaf(A: np.ndarray, B: np.ndarray) -> np.ndarray:
+    """The products in float32, in k order with one fused multiply-add each."""
+    A = np.ascontiguousarray(A, dtype=np.float32)
+    B = np.ascontiguousarray(B, dtype=np.float32)
+    assert A.shape == B.shape and A.shape[-2:] == (64, 64)
+    C = np.empty(A.shape, dtype=np.float32)
+    lib().lko_gemm64_fmaf(_p(A), _p(B), _p(C), A.size // 4096)
     return C
 
 

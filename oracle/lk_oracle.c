@@ -69,6 +69,18 @@ void lko_gemm64_f32(const float* A, const float* B, double* C, size_t tiles) {
   }
 }
 
+/* The same in binary32, in k order with one fused multiply-add each
+ * (fmaf: exact product, one rounding): what a float accumulator leaves. */
+void lko_gemm64_fmaf(const float* A, const float* B, float* C, size_t tiles) {
+  for (size_t t = 0; t < tiles; ++t)
+    for (int i = 0; i < 64; ++i)
+      for (int j = 0; j < 64; ++j) {
+        float s = 0.0f;
+        for (int k = 0; k < 64; ++k) s = fmaf(A[t * 4096 + i * 64 + k], B[t * 4096 + k * 64 + j], s);
+        C[t * 4096 + i * 64 + j] = s;
+      }
+}
+
 /* bound[i][j] = sum_k |A[i][k] * B[k][j]|: the scale of the per-element
  * acceptance bound for a binary32 GEMM. */
 void lko_gemm64_abs_bound(const float* A, const float* B, double* bound, size_t tiles) {

@@ -33,6 +33,7 @@ void   lko_hist_u8(const uint8_t* x, size_t n, int64_t bins[256]);
 double lko_sum_f32(const float* x, size_t n);
 double lko_abs_sum_f32(const float* x, size_t n);
 void   lko_gemm64_f32(const float* A, const float* B, double* C, size_t tiles);
+void   lko_gemm64_fmaf(const float* A, const float* B, float* C, size_t tiles);
 void   lko_gemm64_abs_bound(const float* A, const float* B, double* bound, size_t tiles);
 
 /* The compute-bound loop of Sec. III ("a loop of 20k iterations ... no memory

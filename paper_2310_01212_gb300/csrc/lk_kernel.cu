@@ -1019,7 +1019,7 @@ __device__ __forceinline__ void persistent_main(const lk_kargs& a) {
       break;
     }
   }
-  __syncthreads();   /* warp 1's completion word before thread 0 reports the exit */
+  __syncthreads();   /* finite mode: warp 1 has finished the last descriptor before the CTA reports or leaves */
   if (tid == 0) {
     if (master && mailbox) {
       /* completions the host has not consumed through FINISHED yet stay
