@@ -428,8 +428,9 @@ __device__ __forceinline__ void hist_zero(uint32_t* sh, uint32_t words) {
  * What bounds it is the shared-memory pipe: 512 bytes of input cost 16 warp
  * reductions, a 128-bit read per lane (4 wavefronts) and the TMA write of the
  * same bytes (4), 24 clocks or 21.3 bytes a clock.  Measured per SM: 20.4 with
- * HBM idle (38 CTAs), 19 on 152 CTAs (3 x 1 GiB: 5.80 TB/s; with a permute
- * and an add per address, and two copies to clear and read, 16.6 and 5.23).
+ * HBM idle (38 CTAs), 19 on 152 CTAs (3 x 1 GiB in one launch, boot included:
+ * 5.7 TB/s; with a permute and an add per address, and two copies to clear and
+ * read, 16.6 and 5.2).
  * Loads straight into registers instead of through the ring: 21.1 on 38 CTAs,
  * but 5.24 TB/s on 152, too few bytes in flight.  A second copy of the
  * counters only adds clearing and read-out. */
@@ -976,7 +977,8 @@ __device__ __forceinline__ uint32_t gemm_row_split(uint64_t tiles, int S) {
  * The CTA's eight warps split tile k into operand buffer k mod 2, one thread
  * hands it to the tensor core and refills the raw stage, and while those MMAs
  * run every warp stores its part of tile k-1: one barrier per tile.
- * What bounds it is HBM: 3 x 2^15 tiles move 6.57 TB/s once booted, as much as
+ * What bounds it is HBM: 3 x 2^15 tiles move 6.57 TB/s once booted (6.5 with
+ * the boot), as much as
  * the same loads and stores with neither split nor MMAs (6.63).  One SM alone
  * (38 CTAs, HBM idle) takes 2,060 clocks a tile, against 2,275 of its share of
  * HBM: 1,130 for the loads and stores, the rest for the split and the chain
